@@ -72,3 +72,39 @@ def test_zero_field_stays_and_bad_arguments_fail():
         _run_gpu(np.zeros((10, 10), dtype=np.uint32), keys, 1, 5, "hash")  # grid smaller than 17
     with pytest.raises(gp.GpError):
         _run_gpu(act, keys, 1, 5, "hash", batch=100)  # not a multiple of 32
+
+
+def _field(kind, width, height):
+    rng = np.random.default_rng(width * 1000 + height)
+    if kind == "flat":  # every likelihood of a distance ties
+        return np.full((height, width), 7, dtype=np.uint32)
+    if kind == "spikes":  # mostly nothing, few of the largest values
+        act = np.zeros((height, width), dtype=np.uint32)
+        act[rng.random((height, width)) < 0.01] = 0xFFFFFFFF
+        act[rng.random((height, width)) < 0.05] = 3
+        return act
+    return rng.integers(0, 1 << 20, size=(height, width), dtype=np.uint64).astype(np.uint32)
+
+
+@pytest.mark.parametrize("kind", ["flat", "spikes", "noise"])
+@pytest.mark.parametrize("width,height", [(17, 17), (18, 35), (33, 64), (255, 130), (258, 41), (600, 520)])
+def test_pruned_moves_match_oracle(kind, width, height):
+    # the bound on the activity near a cell's tile: fields smaller than the margin, tiles cut at the
+    # field's edge, tiles of 4 to 16 cells; ties and empty neighbourhoods
+    act = _field(kind, width, height)
+    keys = mg.walk_agents(3, 300, width, height)
+    want, _ = W.run(act, keys, 2, 9)
+    for variant in ("naive", "hash"):
+        got, cnt = _run_gpu(act, keys, 2, 9, variant, 96, 64)
+        assert np.array_equal(got, want)
+        assert int(cnt[2]) == 0
+
+
+@pytest.mark.parametrize("steps", [1, 2])
+def test_bound_rule_both_sides(steps):
+    # 2,704 tiles of 160 x 160 cells read are past 64M for one step, within it for two
+    act = _field("noise", 6600, 6600)
+    keys = mg.walk_agents(4, 100, 6600, 6600)
+    want, _ = W.run(act, keys, steps, 3)
+    got, _ = _run_gpu(act, keys, steps, 3, "warp")
+    assert np.array_equal(got, want)
