@@ -267,14 +267,12 @@ gp_status run_partition(gp_ctx* c, Partition& p, const uint32_t* idx, uint64_t n
   a.segment_tris = p.segment_tris;
   a.num_segments = p.num_segments;
   a.seg_cap = p.seg_cap;
-  a.table_slots = next_pow2(2 * (p.max_unique + 96));
-  a.table_bits = log2u(a.table_slots);
   a.seg_starts = p.d_seg;
   a.seg_counts = p.d_seg + (size_t)p.num_segments * p.seg_cap;
   a.starts = p.d_starts;
   a.num_batches = p.d_count;
   a.err = &c->d_rec[kRing].err;  // the record after the draw ring collects partition errors
-  GP_CUDA(c, launch_partition(a, 4, stream));
+  GP_CUDA(c, launch_partition(a, stream));
   return GP_OK;
 }
 

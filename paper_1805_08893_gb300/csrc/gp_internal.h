@@ -81,8 +81,9 @@ struct PartitionArgs {
   uint32_t segment_tris;     // > 0
   uint32_t num_segments;
   uint32_t seg_cap;          // batch-start slots per segment
-  uint32_t table_slots;      // per-warp hash slots (power of two)
+  uint32_t table_slots;      // hash slots (power of two) and their log2, set by launch_partition
   uint32_t table_bits;
+  uint32_t panel_bits;       // log2 of the triangles per panel of the index ring, set by launch_partition
   uint32_t* seg_starts;      // [num_segments * seg_cap]
   uint32_t* seg_counts;      // [num_segments]
   uint32_t* starts;          // out: [total + 1]
@@ -111,8 +112,7 @@ int reuse_blocks_per_sm(int dedup, bool dynamic, int shader, int threads, size_t
 cudaError_t launch_reuse(int dedup, bool dynamic, bool wide, const DrawArgs& a, const Uniforms& u, int shader,
                          int threads, int grid, size_t smem, cudaStream_t s);
 
-size_t partition_smem_bytes(const PartitionArgs& p, int warps);
-cudaError_t launch_partition(const PartitionArgs& p, int warps_per_block, cudaStream_t s);
+cudaError_t launch_partition(const PartitionArgs& p, cudaStream_t s);
 
 int out_floats(int shader);  // K
 

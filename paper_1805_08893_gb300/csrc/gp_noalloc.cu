@@ -48,12 +48,6 @@ cudaError_t scratch_address(int device, uint32_t** out) {
   *out = g_noalloc_ptr[device];
   return cudaSuccess;
 }
-
-uint32_t next_pow2_u32(uint32_t x) {
-  uint32_t p = 1;
-  while (p < x) p <<= 1;
-  return p;
-}
 }  // namespace
 
 }  // namespace gp
@@ -110,14 +104,11 @@ extern "C" gp_status gp_partition_noalloc(const uint32_t* d_indices, uint64_t nu
   a.segment_tris = seg;
   a.num_segments = nseg;
   a.seg_cap = seg_cap;
-  a.table_slots = next_pow2_u32(2 * (max_unique + 96));
-  a.table_bits = 0;
-  while ((1u << a.table_bits) < a.table_slots) ++a.table_bits;
   a.err = scratch;
   a.seg_starts = scratch + 1;
   a.seg_counts = scratch + 1 + (size_t)nseg * seg_cap;
   a.starts = d_starts;
   a.num_batches = d_num_batches;
-  if ((e = launch_partition(a, 4, s)) != cudaSuccess) return cuda_err("partition launch", e);
+  if ((e = launch_partition(a, s)) != cudaSuccess) return cuda_err("partition launch", e);
   return GP_OK;
 }
