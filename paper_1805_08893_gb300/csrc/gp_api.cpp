@@ -141,15 +141,16 @@ gp_status fold(gp_ctx* c, uint64_t upto) {
   // the records of the folded tickets are consecutive ring slots (maybe wrapping)
   {
     const uint32_t first = c->inflight.front().slot;
-    uint64_t n = 0;
-    for (const Ticket& t : c->inflight)
-      if (t.id <= upto) ++n;
+    const uint64_t n = std::min<uint64_t>(std::min(upto, c->inflight.back().id) - c->inflight.front().id + 1, kRing);
     const uint32_t run1 = (uint32_t)std::min<uint64_t>(n, kRing - first);
     GP_CUDA(c, cudaMemcpyAsync(c->h_rec + first, c->d_rec + first, sizeof(DevRec) * run1, cudaMemcpyDeviceToHost,
                                c->aux));
     if (n > run1)
       GP_CUDA(c, cudaMemcpyAsync(c->h_rec, c->d_rec, sizeof(DevRec) * (n - run1), cudaMemcpyDeviceToHost, c->aux));
     GP_CUDA(c, cudaMemcpyAsync(c->h_rec + kRing, c->d_rec + kRing, sizeof(DevRec), cudaMemcpyDeviceToHost, c->aux));
+    // their next users find them empty (one memset for all of them rather than one per draw)
+    GP_CUDA(c, cudaMemsetAsync(c->d_rec + first, 0, sizeof(DevRec) * run1, c->aux));
+    if (n > run1) GP_CUDA(c, cudaMemsetAsync(c->d_rec, 0, sizeof(DevRec) * (n - run1), c->aux));
     GP_CUDA(c, cudaStreamSynchronize(c->aux));
     if (c->h_rec[kRing].err) worst = fail(c, GP_ERR_UNSUPPORTED, "the dynamic partition exceeded a capacity");
   }
@@ -493,9 +494,17 @@ gp_status check_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* vb,
 }
 
 gp_status new_ticket(gp_ctx* c, Ticket& t) {
-  // a free device record: fold the oldest draw if the ring is full
+  // a free device record: if the ring is full, fold every draw that has completed (their events complete in
+  // order), at least the oldest.  Folding one at a time cost a read-back and a wait of ~15 us per draw.
   if (c->inflight.size() >= kRing) {
-    gp_status s = sync_locked(c, c->inflight.front().id, 0);
+    size_t lo = 0, hi = c->inflight.size();  // draws [0, lo) have completed, draw hi (if any) has not
+    while (lo < hi) {
+      const size_t mid = (lo + hi) / 2;
+      if (cudaEventQuery(c->inflight[mid].ev1) == cudaSuccess) lo = mid + 1;
+      else hi = mid;
+    }
+    cudaGetLastError();  // not ready, or an error that the wait below reports
+    gp_status s = sync_locked(c, c->inflight[lo ? lo - 1 : 0].id, 0);
     if (s != GP_OK && s != GP_ERR_INDEX_RANGE) return s;
   }
   t.id = c->next_ticket++;
@@ -523,11 +532,17 @@ gp_status submit_locked(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* 
   if (s != GP_OK) return s;
   DevRec* rec = c->d_rec + t.slot;
   GP_CUDA(c, cudaEventRecord(t.ev0, c->stream));
-  GP_CUDA(c, cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream));
+  // the record is empty (gp_create, fold), but a captured draw runs more than once
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+  if (cap != cudaStreamCaptureStatusNone) GP_CUDA(c, cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream));
   s = enqueue_draw(c, ib, vb, shader, u, ob, t, rec, pre);
   if (s != GP_OK) {
     put_event(c, t.ev0);
     put_event(c, t.ev1);
+    // the id and its slot go to the next draw, the record empty whatever has run
+    cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream);
+    c->next_ticket = t.id;
     return s;
   }
   GP_CUDA(c, cudaEventRecord(t.ev1, c->stream));
@@ -604,7 +619,8 @@ gp_status gp_create(const gp_config* cfg_in, gp_ctx** out) {
   if ((e = cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaMalloc(&c->d_rec, sizeof(DevRec) * (kRing + 1))) != cudaSuccess ||
       (e = cudaMallocHost(&c->h_rec, sizeof(DevRec) * (kRing + 1))) != cudaSuccess ||
-      (e = cudaMemset(c->d_rec, 0, sizeof(DevRec) * (kRing + 1))) != cudaSuccess) {
+      (e = cudaMemsetAsync(c->d_rec, 0, sizeof(DevRec) * (kRing + 1), c->aux)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(c->aux)) != cudaSuccess) {
     gp_status s = fail(nullptr, e == cudaErrorMemoryAllocation ? GP_ERR_OOM : GP_ERR_CUDA, cudaGetErrorString(e));
     gp_destroy(c);
     return s;

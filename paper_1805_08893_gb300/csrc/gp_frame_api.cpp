@@ -339,9 +339,15 @@ gp_status frame_submit_locked(gp_frame* f, uint64_t* out_ticket) {
   Ticket t;
   gp_status s = new_ticket(c, t);
   if (s != GP_OK) return s;
-  GP_CUDA(c, cudaEventRecord(t.ev0, c->stream));
-  GP_CUDA(c, cudaGraphLaunch(f->exec, c->stream));
-  GP_CUDA(c, cudaEventRecord(t.ev1, c->stream));
+  cudaError_t e = cudaEventRecord(t.ev0, c->stream);
+  if (e == cudaSuccess) e = cudaGraphLaunch(f->exec, c->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(t.ev1, c->stream);
+  if (e != cudaSuccess) {
+    put_event(c, t.ev0);
+    put_event(c, t.ev1);
+    c->next_ticket = t.id;  // the id and its slot go to the next ticket
+    return cuda_fail(c, e, "frame launch");
+  }
   t.draws = f->desc.size();
   t.tris = f->tris;
   t.indices = f->indices;

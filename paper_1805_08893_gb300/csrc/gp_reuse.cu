@@ -686,9 +686,13 @@ size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads) {
   return reuse_layout(dedup, shader, a, (uint32_t)threads).total;
 }
 
+constexpr size_t kMaxDynSmem = 227 * 1024;  // per block, opted in
+
 static int blocks_per_sm(const void* fn, int threads, size_t smem) {
   if (fn == nullptr) return 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  // the limit is the device's, whatever this draw needs: other contexts launch the same function, and
+  // launch_reuse then has nothing to set
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem) != cudaSuccess) return 0;
   cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess) return 0;
@@ -706,9 +710,6 @@ cudaError_t launch_reuse(int dedup, bool dynamic, bool wide, const DrawArgs& a, 
                          int threads, int grid, size_t smem, cudaStream_t s) {
   const void* fn = reuse_kernel_ptr(dedup, dynamic, shader, wide);
   if (fn == nullptr) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   void* args[] = {const_cast<DrawArgs*>(&a), const_cast<Uniforms*>(&u)};
   return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, s);
 }
