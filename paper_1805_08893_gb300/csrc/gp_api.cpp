@@ -436,35 +436,53 @@ gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* v
     const uint32_t pb = std::max(1u, log2u(a.sort_n));
     a.sort_pos_bits = (pb < 32 && (uint64_t)a.num_verts + 1 < (1ull << (32 - pb))) ? pb : 0u;
   }
+  a.row_cap = a.ucap;
   // the kernel splits its block into producer and consumer warps: at least two warps
   const uint32_t block = std::max(64u, threads);
-  const size_t smem = reuse_smem_bytes(dedup, (int)shader, a, (int)block);
+  size_t smem = reuse_smem_bytes(dedup, (int)shader, a, (int)block);
   if (smem > 227 * 1024)
     return fail(c, GP_ERR_UNSUPPORTED, "batch configuration needs more than 227 KB of shared memory");
+  // a static draw's smaller configuration, where more blocks of it fit an SM
+  DrawArgs small = a;
+  const bool can_shrink = !dyn && c->spill_blocks && reuse_shrink_static(small, cfg.hash_slots != 0);
+  const size_t small_smem = can_shrink ? reuse_smem_bytes(dedup, (int)shader, small, (int)block) : 0;
   const uint64_t key = (2ull << 56) | ((uint64_t)dedup << 48) | ((uint64_t)dyn << 47) | ((uint64_t)shader << 40) |
                        ((uint64_t)threads << 24) | (uint64_t)smem;  // smem < 2^24
-  int bpsm;
-  bool wide = false;
+  struct Occ {
+    int bpsm;
+    bool wide, shrink;
+  } occ{};
   auto it = c->occ.find(key);
   if (it != c->occ.end()) {
-    bpsm = it->second & 0xFF;
-    wide = (it->second >> 8) != 0;
+    occ = Occ{it->second & 0xFF, (it->second & 0x100) != 0, (it->second & 0x200) != 0};
   } else {
-    bpsm = reuse_blocks_per_sm(dedup, dyn, (int)shader, (int)block, smem, &wide);
-    c->occ[key] = bpsm | (wide ? 0x100 : 0);
+    occ.bpsm = reuse_blocks_per_sm(dedup, dyn, (int)shader, (int)block, smem, &occ.wide);
+    if (can_shrink && occ.bpsm > 0) {
+      bool wide = false;
+      const int nb = std::min<int>(reuse_blocks_per_sm(dedup, dyn, (int)shader, (int)block, small_smem, &wide),
+                                   (int)(c->spill_blocks / c->sms));
+      if (nb > occ.bpsm) occ = Occ{nb, wide, true};
+    }
+    c->occ[key] = occ.bpsm | (occ.wide ? 0x100 : 0) | (occ.shrink ? 0x200 : 0);
   }
-  if (bpsm <= 0) return fail(c, GP_ERR_UNSUPPORTED, "draw kernel cannot be resident with this configuration");
-  uint64_t grid = (uint64_t)c->sms * bpsm;
+  if (occ.bpsm <= 0) return fail(c, GP_ERR_UNSUPPORTED, "draw kernel cannot be resident with this configuration");
+  if (occ.shrink) {
+    a = small;
+    a.spill = c->d_spill;
+    smem = small_smem;
+  }
+  uint64_t grid = (uint64_t)c->sms * occ.bpsm;
   if (!dyn) grid = std::min<uint64_t>(grid, a.num_batches);
   if (std::getenv("GP_VERBOSE") && c->logged.insert(key).second)
-    std::fprintf(stderr, "[gp] reuse dedup=%d dyn=%d shader=%u threads=%u smem=%zu blocks/SM=%d grid=%llu slots=%u regs=%d\n",
-                 dedup, (int)dyn, shader, block, smem, bpsm, (unsigned long long)grid, a.hash_slots, wide ? 80 : 64);
+    std::fprintf(stderr, "[gp] reuse dedup=%d dyn=%d shader=%u threads=%u smem=%zu blocks/SM=%d grid=%llu slots=%u rows=%u regs=%d\n",
+                 dedup, (int)dyn, shader, block, smem, occ.bpsm, (unsigned long long)grid, a.hash_slots, a.row_cap,
+                 occ.wide ? 80 : 64);
   if (c->test_stall_draws) {  // failure injection: this draw's bounded window wait runs out
     --c->test_stall_draws;
     a.test_stall = 1;
   }
   t.device_counts = true;
-  GP_CUDA(c, launch_reuse(dedup, dyn, wide, a, u, (int)shader, (int)block, (int)std::max<uint64_t>(grid, 1), smem,
+  GP_CUDA(c, launch_reuse(dedup, dyn, occ.wide, a, u, (int)shader, (int)block, (int)std::max<uint64_t>(grid, 1), smem,
                           c->stream));
   return GP_OK;
 }
@@ -625,6 +643,26 @@ gp_status gp_create(const gp_config* cfg_in, gp_ctx** out) {
     gp_destroy(c);
     return s;
   }
+  if (cfg.variant >= GP_SORT && cfg.variant <= GP_PHASH && cfg.mode == GP_BATCH_STATIC) {
+    // room for the static draws' smaller configuration (without it they run with all their rows in shared memory)
+    DrawArgs a{};
+    a.max_batch_idx = a.ucap = cfg.batch_indices;
+    a.hash_slots = cfg.hash_slots ? cfg.hash_slots : 1u << 15;
+    a.sort_n = next_pow2(a.ucap);
+    a.sort_pos_bits = 1;
+    if (reuse_shrink_static(a, cfg.hash_slots != 0)) {
+      const int dedup = cfg.variant == GP_SORT ? DEDUP_SORT : DEDUP_HASH;
+      const size_t smem = reuse_smem_bytes(dedup, GP_SHADER_MVP, a, (int)std::max(64u, th));
+      const uint32_t blocks = (uint32_t)c->sms * (uint32_t)std::min<size_t>(4, 227 * 1024 / smem);
+      void* p = nullptr;
+      if (blocks && cudaMalloc(&p, (size_t)blocks * 4 * (a.ucap - a.row_cap) * sizeof(float4)) == cudaSuccess) {
+        c->d_spill = static_cast<float4*>(p);
+        c->spill_blocks = blocks;
+      } else {
+        cudaGetLastError();
+      }
+    }
+  }
   *out = c;
   return GP_OK;
 }
@@ -650,6 +688,7 @@ gp_status gp_destroy(gp_ctx* c) {
     if (c->h_vtx) cudaFree(c->h_vtx);
     if (c->h_out) cudaFree(c->h_out);
     if (c->d_shaded) cudaFree(c->d_shaded);
+    if (c->d_spill) cudaFree(c->d_spill);
     if (c->copy_in) cudaStreamDestroy(c->copy_in);
     if (c->copy_out) cudaStreamDestroy(c->copy_out);
     if (c->part_stream) cudaStreamDestroy(c->part_stream);

@@ -83,7 +83,7 @@ __device__ __forceinline__ void mvp_transform(const Uniforms& u, float px, float
 }
 
 // Shades one vertex into o[0..K).  'palette' is the skinning palette in
-// shared memory (64 x 12 floats) for SH == 1, unused otherwise.
+// shared memory (64 x 12 floats, 16-byte aligned) for SH == 1, unused otherwise.
 template <int SH>
 __device__ __forceinline__ void shade_vertex(const Uniforms& u, const float* palette, const VertexIn& v,
                                              float* o) {
@@ -94,7 +94,10 @@ __device__ __forceinline__ void shade_vertex(const Uniforms& u, const float* pal
     const float w[4] = {v.w0, v.w1, v.w2, v.w3};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const float* B = palette + 12 * ((v.bones >> (8 * i)) & 0xFFu);
+      // three 16-byte reads: lanes with unrelated bones meet fewer bank conflicts than in twelve of 4
+      const float4* B4 = reinterpret_cast<const float4*>(palette) + 3 * ((v.bones >> (8 * i)) & 0xFFu);
+      const float4 b0 = B4[0], b1 = B4[1], b2 = B4[2];
+      const float B[12] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w, b2.x, b2.y, b2.z, b2.w};
       float t0 = __fmaf_rn(B[0], v.px, __fmaf_rn(B[1], v.py, __fmaf_rn(B[2], v.pz, B[3])));
       float t1 = __fmaf_rn(B[4], v.px, __fmaf_rn(B[5], v.py, __fmaf_rn(B[6], v.pz, B[7])));
       float t2 = __fmaf_rn(B[8], v.px, __fmaf_rn(B[9], v.py, __fmaf_rn(B[10], v.pz, B[11])));

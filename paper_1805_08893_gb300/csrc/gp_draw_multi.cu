@@ -17,7 +17,7 @@ template <int SH>
 __global__ void __launch_bounds__(256) shade_all_kernel(const __grid_constant__ DrawArgs a,
                                                         const __grid_constant__ Uniforms u, float4* rows) {
   constexpr int K = ShaderTraits<SH>::K;
-  __shared__ float palette[ShaderTraits<SH>::kSkin ? 768 : 1];
+  __shared__ __align__(16) float palette[ShaderTraits<SH>::kSkin ? 768 : 1];
   if (ShaderTraits<SH>::kSkin) {
     for (int i = threadIdx.x; i < 768; i += blockDim.x) palette[i] = u.palette[i];
     __syncthreads();

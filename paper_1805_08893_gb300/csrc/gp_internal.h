@@ -38,7 +38,7 @@ struct Uniforms {
   float inv_dirs;        // ENVELOPE: 1 / num_dirs
   float dirs[kMaxEnvelopeDirs * 3];
   float coef[kEnvelopeTerms];  // ENVELOPE: 1/k!, k = 0..31
-  float palette[64 * 12];      // SKIN
+  alignas(16) float palette[64 * 12];  // SKIN (16-byte reads)
 };
 
 // One draw as the kernels see it.
@@ -61,6 +61,9 @@ struct DrawArgs {
   const uint32_t* num_batches_dev;  // dynamic: device batch count
   uint32_t max_batch_idx;        // capacity: indices per batch
   uint32_t ucap;                 // capacity: unique vertices per batch
+  uint32_t row_cap;              // single-draw reuse kernel: vertex rows a batch has in shared memory (<= ucap) ...
+  float4* spill;                 // ... and, static batches, where shaded vertices past them go: 2 x (ucap - row_cap)
+                                 // vertices of two float4 per block
   uint32_t hash_slots;           // power of two
   uint32_t hash_bits;            // log2(hash_slots)
   uint32_t sort_n;               // power of two >= max_batch_idx
@@ -106,6 +109,10 @@ size_t warp_kernel_smem(int shader, int warps_per_block, uint32_t batch_idx);
 
 // Single-draw sort/hash/phash kernel (gp_reuse.cu).
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads);
+// The smaller shared-memory configuration of a static draw (rows for a third
+// of the capacity, a fuller hash table unless the caller chose its size);
+// false: the batch is too small to gain from it.
+bool reuse_shrink_static(DrawArgs& a, bool own_slots);
 // Blocks per SM of the 64-register kernel; *wide: the 80-register kernel
 // exists for this draw and fits as many (launch it instead).
 int reuse_blocks_per_sm(int dedup, bool dynamic, int shader, int threads, size_t smem, bool* wide);

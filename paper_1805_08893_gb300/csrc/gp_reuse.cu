@@ -68,8 +68,9 @@ __host__ __device__ inline uint32_t reuse_producer_warps(uint32_t NT, int dedup)
 // Groups (4 positions) a producer thread inserts per pass, all CAS in flight.
 constexpr int kGroupsPerPass = 2;
 
-// Shared-memory layout for NT threads.  K: floats per output corner.
-__host__ __device__ inline ReuseLayout reuse_layout(int dedup, int shader, const DrawArgs& a, uint32_t NT) {
+// Shared-memory layout for NT threads, row_cap rows a slot (a.row_cap; a.ucap says
+// the same of dynamic batches).  K: floats per output corner.
+__host__ __device__ inline ReuseLayout reuse_layout(int dedup, int shader, const DrawArgs& a, uint32_t NT, uint32_t row_cap) {
   const uint32_t K = shader == 2 ? 8u : 7u;
   const uint32_t consumer_warps = NT / 32 - reuse_producer_warps(NT, dedup);
   ReuseLayout L;
@@ -95,7 +96,7 @@ __host__ __device__ inline ReuseLayout reuse_layout(int dedup, int shader, const
   L.ring_dense = reuse_align16(L.map_elems * 2);
   L.ring_uniq = L.ring_dense + reuse_align16(dedup == DEDUP_SORT ? 0u : a.hash_slots * 2);
   L.ring_rows = L.ring_uniq + L.uniq_words * 4;  // uniq_words is a multiple of 4
-  L.ring_bytes = L.ring_rows + a.ucap * L.rb;     // rows are 32 or 64 bytes
+  L.ring_bytes = L.ring_rows + row_cap * L.rb;    // rows are 32 or 64 bytes
   o += 2 * L.ring_bytes;
   L.off_stage = o; o += consumer_warps * 32 * K * 16;
   L.off_pal = o; o += shader == 1 ? 768 * 4 : 0;
@@ -169,7 +170,7 @@ struct RowCopy {
   unsigned char* rows;
   const uint32_t* uniq;
   __device__ __forceinline__ void operator()(uint32_t rb, uint32_t re, uint32_t lane) const {
-    re = min(re, a.ucap);
+    re = min(re, a.row_cap);
     for (uint32_t r = rb + lane; r < re; r += 32) copy_row<SH>(a, rows, r, uniq[r]);
   }
 };
@@ -181,7 +182,7 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
   extern __shared__ __align__(128) unsigned char smem[];
   const uint32_t tid = threadIdx.x, NT = blockDim.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t NPW = reuse_producer_warps(NT, DEDUP), NP = 32 * NPW, NC = NT - NP;
-  const ReuseLayout L = reuse_layout(DEDUP, SH, a, NT);
+  const ReuseLayout L = reuse_layout(DEDUP, SH, a, NT, DYN ? a.ucap : a.row_cap);
   const uint32_t nb = DYN ? *a.num_batches_dev : a.num_batches;
   if (blockIdx.x >= nb) return;
 
@@ -464,7 +465,7 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
               if (r < a.ucap) {
                 dense[sl[q]] = (uint16_t)r;
                 uniq[r] = id[q];
-                copy_row<SH>(a, rows, r, id[q]);
+                if (DYN || r < a.row_cap) copy_row<SH>(a, rows, r, id[q]);
               } else {
                 atomicOr(a.err, EBIT_CAPACITY);
               }
@@ -525,6 +526,9 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
       unsigned char* rows = slot_p + L.ring_rows;
       float4* vsh = reinterpret_cast<float4*>(rows);
       const uint32_t U = min(misc[s], a.ucap);
+      // where this slot's shaded vertices past row_cap go (a slot's readers are done before its next writers:
+      // the consumers' barrier of the batch between)
+      float4* spill = DYN ? nullptr : a.spill + (size_t)2 * (a.ucap - a.row_cap) * (2 * blockIdx.x + s);
 
       // --- shade each unique vertex once, in place
       for (uint32_t r = ctid; r < U; r += NC) {
@@ -532,7 +536,8 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
         const uint32_t id = uniq[r];
         if (id < a.num_verts) {
           VertexIn v;
-          load_raw<SH>(rows + r * RB, v);
+          if (DYN || r < a.row_cap) load_raw<SH>(rows + r * RB, v);
+          else fetch_vertex<SH>(a.verts, a.stride, id, v, a.vec8 != 0);
           shade_vertex<SH>(u, palette, v, o);
         } else {
 #pragma unroll
@@ -540,8 +545,14 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
           atomicOr(a.err, EBIT_INDEX_RANGE);
         }
         if (K == 7) o[7] = 0.f;
-        vsh[row_slot<SH>(r, 0)] = make_float4(o[0], o[1], o[2], o[3]);
-        vsh[row_slot<SH>(r, 1)] = make_float4(o[4], o[5], o[6], o[7]);
+        const float4 lo = make_float4(o[0], o[1], o[2], o[3]), hi = make_float4(o[4], o[5], o[6], o[7]);
+        if (DYN || r < a.row_cap) {
+          vsh[row_slot<SH>(r, 0)] = lo;
+          vsh[row_slot<SH>(r, 1)] = hi;
+        } else {
+          spill[2 * (r - a.row_cap)] = lo;
+          spill[2 * (r - a.row_cap) + 1] = hi;
+        }
       }
       named_sync(kBarConsumers, NC);  // every unique vertex shaded; every consumer has read the counter
       if (ctid == 0) {
@@ -564,7 +575,14 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
           for (int e = 0; e < 4; ++e) {
             uint32_t r = (DEDUP == DEDUP_SORT) ? sl[e] : (uint32_t)dense[sl[e]];
             r = r < U ? r : 0u;  // positions outside the batch (never written) and flagged capacity errors
-            const float4 lo = vsh[row_slot<SH>(r, 0)], hi = vsh[row_slot<SH>(r, 1)];
+            float4 lo, hi;
+            if (DYN || r < a.row_cap) {
+              lo = vsh[row_slot<SH>(r, 0)];
+              hi = vsh[row_slot<SH>(r, 1)];
+            } else {
+              lo = spill[2 * (r - a.row_cap)];
+              hi = spill[2 * (r - a.row_cap) + 1];
+            }
             if (K == 8) {  // a corner is two whole float4
               stage[stage_put<K>(lane, 2 * e)] = lo;
               stage[stage_put<K>(lane, 2 * e + 1)] = hi;
@@ -682,8 +700,31 @@ static const void* reuse_kernel_ptr(int dedup, bool dyn, int shader, bool wide) 
   }
 }
 
+// Static batches have room for S unique vertices, yet a batch of a mesh with
+// locality holds a fifth to a third of S: with rows (and table) for all of
+// them a 768-index batch takes 98 KB of a block (skinning: 151 KB, one block
+// per SM).  Here the rows are for a third, the ones past it are shaded from
+// global memory into 'spill', and the table may be three quarters full.  On a
+// skinned 500k-triangle mesh: 3 blocks per SM, 38 us against 55.
+bool reuse_shrink_static(DrawArgs& a, bool own_slots) {
+  if (a.ucap < 192) return false;
+  a.row_cap = (a.ucap / 3 + 3) & ~3u;
+  if (!own_slots) {
+    uint32_t slots = 1024, bits = 10;
+    while (slots < a.ucap + a.ucap / 3) {
+      slots <<= 1;
+      ++bits;
+    }
+    if (slots < a.hash_slots) {
+      a.hash_slots = slots;
+      a.hash_bits = bits;
+    }
+  }
+  return true;
+}
+
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads) {
-  return reuse_layout(dedup, shader, a, (uint32_t)threads).total;
+  return reuse_layout(dedup, shader, a, (uint32_t)threads, a.row_cap).total;
 }
 
 constexpr size_t kMaxDynSmem = 227 * 1024;  // per block, opted in
