@@ -33,6 +33,7 @@ struct LoopArgs {
   uint32_t num_tris;
   const unsigned char* verts;
   uint32_t stride, num_verts;
+  uint32_t vec16;                 // 1: rows are 16-byte aligned (one load per position)
   const uint32_t* ring_off;
   const uint32_t* ring;
   uint32_t ring_count;
@@ -53,13 +54,17 @@ __device__ __forceinline__ float3 loop_pos(const LoopArgs& a, uint32_t v) {
     atomicOr(a.counters + 2, (unsigned long long)EBIT_INDEX_RANGE);
     return make_float3(0.f, 0.f, 0.f);
   }
-  const float* p = reinterpret_cast<const float*>(a.verts + (size_t)v * a.stride);
+  const unsigned char* row = a.verts + (size_t)v * a.stride;
+  if (a.vec16) {
+    const float4 x = __ldg(reinterpret_cast<const float4*>(row));
+    return make_float3(x.x, x.y, x.z);
+  }
+  const float* p = reinterpret_cast<const float*>(row);
   return make_float3(__ldg(p), __ldg(p + 1), __ldg(p + 2));
 }
 
-// Loop's vertex rule for vertex v.
-__device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v) {
-  const float3 p = loop_pos(a, v);
+// Loop's vertex rule for vertex v at p.
+__device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v, float3 p) {
   if (v >= a.num_verts) return p;
   // ring entries past the ring array (inconsistent adjacency) are not read
   const uint32_t o0 = min(__ldg(a.ring_off + v), a.ring_count);
@@ -125,8 +130,8 @@ __global__ void __launch_bounds__(256) loop_naive_kernel(const __grid_constant__
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const uint32_t v = __ldg(a.idx + 3 * t + k);
-    E[k] = loop_even(a, v);
     P[k] = loop_pos(a, v);
+    E[k] = loop_even(a, v, P[k]);
   }
   loop_emit(a, t, E, P);
 }
@@ -142,7 +147,7 @@ struct LoopEven {
     re = min(re, ucap);  // ranks >= ucap (a flagged capacity error) were not stored
     for (uint32_t r = rb + lane; r < re; r += 32) {
       const uint32_t v = uniq[r];
-      const float3 e = loop_even(la, v), p = loop_pos(la, v);
+      const float3 p = loop_pos(la, v), e = loop_even(la, v, p);
       esh[3 * r] = e.x; esh[3 * r + 1] = e.y; esh[3 * r + 2] = e.z;
       psh[3 * r] = p.x; psh[3 * r + 1] = p.y; psh[3 * r + 2] = p.z;
     }
@@ -246,8 +251,8 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
       }
       float3 E = make_float3(0.f, 0.f, 0.f), P = E;
       if (lane < fill) {
-        E = loop_even(la, held[lane]);
         P = loop_pos(la, held[lane]);
+        E = loop_even(la, held[lane], P);
       }
       inv += fill;
       const uint32_t tfirst = (B0 + c) / 3;
@@ -324,6 +329,7 @@ extern "C" gp_status gp_loop_subdivide(const gp_loop_desc* d) {
   la.verts = static_cast<const unsigned char*>(d->d_vertices);
   la.stride = d->stride_bytes;
   la.num_verts = (uint32_t)d->num_vertices;
+  la.vec16 = reinterpret_cast<uintptr_t>(d->d_vertices) % 16 == 0 && d->stride_bytes % 16 == 0 ? 1u : 0u;
   la.ring_off = d->d_ring_offsets;
   la.ring = d->d_ring;
   la.ring_count = (uint32_t)std::min<uint64_t>(d->ring_count, 0xFFFFFFFFu);
