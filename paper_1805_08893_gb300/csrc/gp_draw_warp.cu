@@ -1,12 +1,17 @@
 // Statically batched warp voting (Algorithm 1, Section 3.3): one warp per
 // static batch, persistent warps walking the batches with a grid stride.  The
-// per-batch work is warp_vote_batch (gp_warp_body.cuh).
+// per-batch work is warp_vote_batch (gp_warp_body.cuh): a chain of ~10 rounds of
+// votes, scattered row loads and shuffles per three batches, bound by the issue
+// of its instructions and the rows' latency.  1.09M triangles, S = 96: 49 us;
+// written and stored round by round, 56.  At most 80 registers a thread (24
+// warps an SM): at 64 or 48 the spills cost more (60 us), without a limit the
+// kernel takes 140 (66 us).
 #include "gp_warp_body.cuh"
 
 namespace gp {
 
 template <int SH>
-__global__ void __launch_bounds__(256) warp_kernel(const __grid_constant__ DrawArgs a,
+__global__ void __launch_bounds__(256, 3) warp_kernel(const __grid_constant__ DrawArgs a,
                                                    const __grid_constant__ Uniforms u) {
   using L = WarpSmem<SH>;
   constexpr int K = L::K;
@@ -24,13 +29,16 @@ __global__ void __launch_bounds__(256) warp_kernel(const __grid_constant__ DrawA
 
   const uint32_t warps_total = gridDim.x * (blockDim.x >> 5);
   unsigned long long inv_total = 0, batches = 0;
+  WarpState st;
+  st.load(a, blockIdx.x * (blockDim.x >> 5) + warp, lane);
   for (uint32_t b = blockIdx.x * (blockDim.x >> 5) + warp; b < a.num_batches; b += warps_total) {
-    const uint32_t inv = warp_vote_batch<SH>(a, u, palette, b, wp, lane);
+    const uint32_t inv = warp_vote_batch<SH>(a, u, palette, b, b + warps_total, wp, lane, st);
     if (lane == 0 && a.batch_inv != nullptr && b < a.batch_cap) a.batch_inv[b] = inv;
     inv_total += inv;
     batches += 1;
     __syncwarp();
   }
+  st.settle(lane);  // the block's shared memory must outlive the last copy
   if (lane == 0 && batches) {
     atomicAdd(a.counters + CNT_INVOCATIONS, inv_total);
     atomicAdd(a.counters + CNT_BATCHES, batches);

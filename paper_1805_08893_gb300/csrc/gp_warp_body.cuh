@@ -44,13 +44,20 @@ __device__ __forceinline__ void warp_vote_round(const uint32_t* widx, uint32_t n
                                                 unsigned char* map, uint32_t lane, uint32_t& fill_out,
                                                 uint32_t& done_out) {
   uint32_t fill = 0, done = 0, off = c;
+  held[lane] = kEmpty;  // no valid id; lanes not yet held compare unequal
+  __syncwarp();
   while (off < n && fill < 32) {
     const uint32_t pos = off + lane;
     const bool valid = pos < n;
     const uint32_t x = valid ? widx[pos] : kEmpty;
-    int hs = -1;  // lane already holding x (earlier chunks of the round)
-    for (uint32_t h = 0; h < fill; ++h)
-      if (held[h] == x) hs = (int)h;
+    int hs = -1;  // lane already holding x (earlier chunks of the round); four ids per read
+    for (uint32_t h = 0; h < fill; h += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(held + h);
+      if (v.x == x) hs = (int)h;
+      if (v.y == x) hs = (int)h + 1;
+      if (v.z == x) hs = (int)h + 2;
+      if (v.w == x) hs = (int)h + 3;
+    }
     const uint32_t grp = __match_any_sync(kFull, x);
     const uint32_t leader = __ffs(grp) - 1;
     const bool is_new = valid && hs < 0 && leader == lane;
@@ -72,11 +79,45 @@ __device__ __forceinline__ void warp_vote_round(const uint32_t* widx, uint32_t n
   done_out = done;
 }
 
+// A warp's state across the batches it processes: the next batch's indices,
+// read one batch ahead (batches of at most kWarpAhead indices), and whether a
+// bulk store may still read its staging area.
+constexpr uint32_t kWarpAhead = 96;
+
+struct WarpState {
+  uint32_t ids[kWarpAhead / 32];
+  bool pending = false;
+
+  __device__ __forceinline__ void load(const DrawArgs& a, uint32_t b, uint32_t lane) {
+    const uint32_t S = 3u * a.static_batch_tris;
+    if (S > kWarpAhead) return;
+#pragma unroll
+    for (uint32_t q = 0; q < kWarpAhead / 32; ++q) {
+      const uint32_t i = 32 * q + lane;
+      const uint64_t at = (uint64_t)b * S + i;
+      ids[q] = i < S && at < a.num_idx ? __ldg(a.idx + at) : 0u;
+    }
+  }
+  // Before the staging area is written again.
+  __device__ __forceinline__ void settle(uint32_t lane) {
+    if (pending) {
+      if (lane == 0) bulk_wait_read<0>();
+      __syncwarp();
+      pending = false;
+    }
+  }
+};
+
 // Processes static batch b (indices [b*S, min((b+1)*S, 3T))) with the warp's
-// shared memory at wp; returns the shader invocations.
+// shared memory at wp; returns the shader invocations.  st.load has read the
+// batch's indices; 'next' is the batch to read ahead.
+// A batch of at most 32 triangles that starts on a 16-byte boundary of the
+// output is assembled whole in the staging area, round by round, and leaves in
+// one bulk store; larger ones are written round by round.
 template <int SH>
 __device__ __forceinline__ uint32_t warp_vote_batch(const DrawArgs& a, const Uniforms& u, const float* palette,
-                                                    uint32_t b, unsigned char* wp, uint32_t lane) {
+                                                    uint32_t b, uint32_t next, unsigned char* wp, uint32_t lane,
+                                                    WarpState& st) {
   using L = WarpSmem<SH>;
   constexpr int K = L::K;
   constexpr int F = L::F;
@@ -88,10 +129,19 @@ __device__ __forceinline__ uint32_t warp_vote_batch(const DrawArgs& a, const Uni
   const uint32_t B0 = b * S;
   const uint32_t B1 = min(B0 + S, a.num_idx);
   const uint32_t n = B1 - B0;
-  for (uint32_t i = lane; i < n; i += 32) {
-    uint32_t id = __ldg(a.idx + B0 + i);
-    widx[i] = id < a.num_verts ? id : kInvalidId;
+  if (S <= kWarpAhead) {
+#pragma unroll
+    for (uint32_t q = 0; q < kWarpAhead / 32; ++q)
+      if (32 * q + lane < n) widx[32 * q + lane] = st.ids[q] < a.num_verts ? st.ids[q] : kInvalidId;
+    st.load(a, next, lane);
+  } else {
+    for (uint32_t i = lane; i < n; i += 32) {
+      const uint32_t id = __ldg(a.idx + B0 + i);
+      widx[i] = id < a.num_verts ? id : kInvalidId;
+    }
   }
+  const size_t out0 = (size_t)B0 * K;  // first float of the batch
+  const bool whole = n <= 96 && (out0 & 3) == 0 && ((n * K) & 3) == 0;
   __syncwarp();
   uint32_t inv = 0;
   uint32_t c = 0;  // round start, relative to B0
@@ -111,38 +161,48 @@ __device__ __forceinline__ uint32_t warp_vote_batch(const DrawArgs& a, const Uni
       for (int k = 0; k < K; ++k) v[k] = 0.f;
     }
     inv += fill;
+    st.settle(lane);
     // emit triangles [ (B0 + c)/3, +tris ) in passes of up to 32 triangles
-    const uint32_t tfirst = (B0 + c) / 3;
     for (uint32_t p = 0; p < tris; p += 32) {
       const uint32_t np = min(32u, tris - p);
-      const size_t g0 = (size_t)(tfirst + p) * F;
+      const size_t g0 = out0 + (size_t)(c + 3 * p) * K;
       const uint32_t pad = (uint32_t)(g0 & 3);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const uint32_t cc = q * 32 + lane;
+      float* to = whole ? stage + c * K : stage + pad;
+#pragma unroll 1
+      for (uint32_t cq = 0; cq < 3 * np; cq += 32) {  // seldom more than once: a round has about 10 triangles
+        const uint32_t cc = cq + lane;
         const bool live = cc < 3 * np;
         const uint32_t s = live ? map[3 * p + cc] : 0u;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
           const float val = __shfl_sync(kFull, v[k], s);
-          if (live) stage[pad + cc * K + k] = val;
+          if (live) to[cc * K + k] = val;
         }
         if (live && a.corner_ids != nullptr) a.corner_ids[B0 + c + 3 * p + cc] = held[s];
       }
       __syncwarp();
+      if (whole) continue;
       const uint32_t nfl = np * F;
       const uint32_t head = min(nfl, (4u - pad) & 3u);
       float* dst = a.out + g0;
-      const float* src = stage + pad;
-      if (lane < head) dst[lane] = src[lane];
+      if (lane < head) dst[lane] = to[lane];
       const uint32_t n4 = (nfl - head) >> 2;
       float4* d4 = reinterpret_cast<float4*>(dst + head);
-      const float4* s4 = reinterpret_cast<const float4*>(src + head);
+      const float4* s4 = reinterpret_cast<const float4*>(to + head);
       for (uint32_t i = lane; i < n4; i += 32) __stcs(d4 + i, s4[i]);
-      for (uint32_t i = head + (n4 << 2) + lane; i < nfl; i += 32) dst[i] = src[i];
+      for (uint32_t i = head + (n4 << 2) + lane; i < nfl; i += 32) dst[i] = to[i];
       __syncwarp();
     }
     c += 3 * tris;
+  }
+  if (whole) {
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      bulk_store(a.out + out0, stage, n * K * 4);
+      bulk_commit();
+    }
+    st.pending = true;
   }
   return inv;
 }
