@@ -342,10 +342,11 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
             uint4 w = make_uint4(0, 0, 0, 0);
             if (g < ngroups) w = reinterpret_cast<const uint4*>(win)[g];
             const uint32_t raw[4] = {w.x, w.y, w.z, w.w};
+            // positions [pad, pad + n) of the window: all four of a group but at its two ends
+            const uint32_t hi = min(pad + n - min(4 * g, pad + n), 4u), lo = g == 0 ? pad : 0u;
+            act |= (((1u << hi) - 1u) & ~((1u << lo) - 1u)) << (4 * k);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              const uint32_t p = 4 * g + e;
-              act |= (g < ngroups && p >= pad && p < pad + n ? 1u : 0u) << (4 * k + e);
               id[4 * k + e] = raw[e] < a.num_verts ? raw[e] : kInvalidId;
               sl[4 * k + e] = hash_slot(id[4 * k + e], a.hash_bits);
             }
@@ -353,8 +354,10 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
           // the first probe of every position, issued before any result is used
 #pragma unroll
           for (int q = 0; q < Q; ++q) prev[q] = (act >> q) & 1u ? atomicCAS(&tbl[sl[q]], kEmpty, id[q]) : kEmpty;
-          // resolve collisions: every position still probing advances one
-          // slot per round, the round's CAS all in flight together
+          // collisions (6% of the positions at the tuned limits): a thread's
+          // positions still probing are taken up one after another, a slot at a
+          // time, in one loop -- advancing all eight together takes as many
+          // rounds as the longest chain of the warp, ~90 instructions each
           uint32_t probing = 0;
 #pragma unroll
           for (int q = 0; q < Q; ++q) {
@@ -362,33 +365,36 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
             else if (prev[q] == kEmpty) newmask |= 1u << q;
             else if (prev[q] != id[q]) probing |= 1u << q;
           }
-          const uint32_t rounds = DEDUP == DEDUP_HASH ? a.hash_slots : a.probe_k;  // per-thread probes
-          for (uint32_t round = 1; probing && round < rounds; ++round) {
+          const uint32_t most = DEDUP == DEDUP_HASH ? a.hash_slots : a.probe_k;  // per-thread probes of a position
+          for (uint32_t tries = 1; probing;) {
+            const uint32_t q = __ffs(probing) - 1;
+            uint32_t myid = id[0], at = sl[0];
 #pragma unroll
-            for (int q = 0; q < Q; ++q)
-              if ((probing >> q) & 1u) {
-                sl[q] = (sl[q] + 1) & mask;
-                prev[q] = atomicCAS(&tbl[sl[q]], kEmpty, id[q]);
+            for (int k = 1; k < Q; ++k)
+              if (q == (uint32_t)k) {
+                myid = id[k];
+                at = sl[k];
               }
-#pragma unroll
-            for (int q = 0; q < Q; ++q)
-              if ((probing >> q) & 1u) {
-                if (prev[q] == kEmpty) newmask |= 1u << q;
-                if (prev[q] == kEmpty || prev[q] == id[q]) probing &= ~(1u << q);
-              }
-          }
-          if (DEDUP == DEDUP_HASH) {
-            if (probing) {  // table full: cannot happen within capacity
+            at = (at + 1) & mask;
+            bool over = tries >= most;  // alone no further: the next slot to probe is 'at'
+            uint32_t got = 0;
+            if (!over) {
+              got = atomicCAS(&tbl[at], kEmpty, myid);
+              ++tries;
+              newmask |= (got == kEmpty ? 1u : 0u) << q;
+            } else if (DEDUP == DEDUP_HASH) {  // table full: cannot happen within capacity
               atomicOr(a.err, EBIT_CAPACITY);
-#pragma unroll
-              for (int q = 0; q < Q; ++q)
-                if ((probing >> q) & 1u) sl[q] = 0;
+              at = 0;
+            } else {
+              pend |= 1u << q;
             }
-          } else {
 #pragma unroll
-            for (int q = 0; q < Q; ++q)
-              if ((probing >> q) & 1u) sl[q] = (sl[q] + 1) & mask;  // the next slot to probe
-            pend = probing;
+            for (int k = 0; k < Q; ++k)
+              if (q == (uint32_t)k) sl[k] = at;
+            if (over || got == kEmpty || got == myid) {
+              probing &= probing - 1;
+              tries = 1;
+            }
           }
           if (DEDUP == DEDUP_PHASH) {
             // the positions still pending (rare), one at a time -- the lowest
@@ -459,18 +465,33 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
           if (lane == 0 && total) r = atomicAdd(counter, total);
           r = __shfl_sync(kFull, r, 0) + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt) +
               8 * __popc(b3 & lt);
+          // With the envelope shader, whose producers wait for the consumers, a
+          // warp's new rows are copied one per lane (a lane holds one new id of
+          // every five positions): fewer instructions for the other role,
+          // 103.8 -> 100.9 us on 2M triangles.  Elsewhere each row starts as
+          // soon as its id is known: 198.6 us against 204.2 on the 7.2M-triangle mesh.
+          constexpr bool kGather = SH == 2;
+          uint32_t rw = 0;  // the warp's first rank
+          if constexpr (kGather) rw = __shfl_sync(kFull, r, 0);
 #pragma unroll
           for (int q = 0; q < Q; ++q) {
             if ((newmask >> q) & 1u) {
               if (r < a.ucap) {
                 dense[sl[q]] = (uint16_t)r;
                 uniq[r] = id[q];
-                if (DYN || r < a.row_cap) copy_row<SH>(a, rows, r, id[q]);
+                if constexpr (!kGather) {
+                  if (DYN || r < a.row_cap) copy_row<SH>(a, rows, r, id[q]);
+                }
               } else {
                 atomicOr(a.err, EBIT_CAPACITY);
               }
               ++r;
             }
+          }
+          if constexpr (kGather) {
+            __syncwarp();
+            const uint32_t re = min(rw + total, DYN ? a.ucap : a.row_cap);
+            for (uint32_t k = rw + lane; k < re; k += 32) copy_row<SH>(a, rows, k, uniq[k]);
           }
 #pragma unroll
           for (int k = 0; k < kGroupsPerPass; ++k) {
