@@ -154,61 +154,86 @@ __device__ __forceinline__ void load_raw(const unsigned char* row, VertexIn& v) 
 // lie in one run (ascending where (E tid) & k == 0), and for j >= E they are
 // all on the same side of their pairs, so direction and side are worked out
 // once per stage; each exchange is then a min or a max.
-// The network on keys already in registers (r: keys E tid .. E tid + E - 1);
-// the shared-memory stages use keys[0..N) as their exchange buffer.  Leaves
-// the sorted keys in r.
+// One exchange stage of distance j of the network on keys already in registers
+// (r: keys E tid .. E tid + E - 1); 'up' (k >= E: the thread's run ascends) and
+// the shared-memory exchange buffer keys[0..N) as below.
 template <int E, class T, class Sync>
-__device__ __forceinline__ void bitonic_network_regs(T (&r)[E], T* keys, uint32_t N, uint32_t tid, Sync sync) {
+__device__ __forceinline__ void bitonic_stage_regs(T (&r)[E], T* keys, uint32_t k, uint32_t j, bool up, uint32_t tid,
+                                                   Sync sync) {
   const uint32_t i0 = E * tid;  // this thread's first key
-  for (uint32_t k = 2; k <= N; k <<= 1) {
-    const bool asc = (i0 & k) == 0;  // the thread's run (k >= E)
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      if (j >= (uint32_t)E) {
-        const bool take_min = ((i0 & j) == 0) == asc;  // lower side of an ascending pair, or upper of a descending
-        if (j >= 32u * E) {
-          sync();  // every thread has read the previous contents
+  if (j >= (uint32_t)E) {
+    const bool take_min = ((i0 & j) == 0) == up;  // lower side of an ascending pair, or upper of a descending
+    if (j >= 32u * E) {
+      sync();  // every thread has read the previous contents
 #pragma unroll
-          for (int e = 0; e < E; ++e) keys[i0 + e] = r[e];
-          sync();
+      for (int e = 0; e < E; ++e) keys[i0 + e] = r[e];
+      sync();
 #pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const T y = keys[(i0 + e) ^ j];
-            r[e] = take_min ? (r[e] < y ? r[e] : y) : (r[e] < y ? y : r[e]);
-          }
-        } else {
-          const uint32_t lm = j / E;
+      for (int e = 0; e < E; ++e) {
+        const T y = keys[(i0 + e) ^ j];
+        r[e] = take_min ? (r[e] < y ? r[e] : y) : (r[e] < y ? y : r[e]);
+      }
+    } else {
 #pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const T y = __shfl_xor_sync(kFull, r[e], lm);
-            r[e] = take_min ? (r[e] < y ? r[e] : y) : (r[e] < y ? y : r[e]);
-          }
-        }
-      } else {
-        // j < E: both keys of a pair are in this thread (j is 1, 2 or 4, each
-        // with compile-time register indices); the lower one keeps the
-        // smaller key in an ascending run
-        auto exch = [&](int lo, int hi) {
-          const bool up = k >= (uint32_t)E ? asc : ((i0 + lo) & k) == 0;
-          const T a = r[lo], b = r[hi];
-          const T mn = a < b ? a : b, mx = a < b ? b : a;
-          r[lo] = up ? mn : mx;
-          r[hi] = up ? mx : mn;
-        };
-        if (j == 1) {
-#pragma unroll
-          for (int e = 0; e < E; e += 2) exch(e, e + 1);
-        } else if (j == 2) {
-#pragma unroll
-          for (int e = 0; e < E; ++e)
-            if ((e & 2) == 0) exch(e, e + 2);
-        } else {
-#pragma unroll
-          for (int e = 0; e < E; ++e)
-            if ((e & 4) == 0 && e + 4 < E) exch(e, e + 4);
-        }
+      for (int e = 0; e < E; ++e) {
+        const T y = __shfl_xor_sync(kFull, r[e], j / E);
+        r[e] = take_min ? (r[e] < y ? r[e] : y) : (r[e] < y ? y : r[e]);
       }
     }
+  } else {
+    // j < E: both keys of a pair are in this thread; the lower one keeps the
+    // smaller key in an ascending run
+#pragma unroll
+    for (int lo = 0; lo < E; ++lo)
+      if ((lo & j) == 0) {
+        const int hi = (lo + j) & (E - 1);
+        const bool asc = k >= (uint32_t)E ? up : (lo & k) == 0;
+        const T x = r[lo], y = r[hi];
+        const T mn = x < y ? x : y, mx = x < y ? y : x;
+        r[lo] = asc ? mn : mx;
+        r[hi] = asc ? mx : mn;
+      }
   }
+}
+
+// The network on keys already in registers; the shared-memory stages use
+// keys[0..N) as their exchange buffer.  Leaves the sorted keys in r.
+// 32-bit keys: the stages up to k = 1024 are unrolled, so that distances and
+// register numbers are constants, and the keys of a descending run are kept
+// complemented, so that every thread's run ascends: an exchange inside the
+// thread is a plain min and max.  A 1024-key sort on 128 threads, four blocks
+// per SM: 2,360 cycles of the SM; unrolled without the complements 2,600; one
+// loop over all stages 3,660.
+template <int E, class T, class Sync>
+__device__ __forceinline__ void bitonic_network_regs(T (&r)[E], T* keys, uint32_t N, uint32_t tid, Sync sync) {
+  const uint32_t i0 = E * tid;
+  uint32_t k0 = 2;
+  if (sizeof(T) == 4) {
+    T flip = 0;  // this thread's complement
+#pragma unroll
+    for (uint32_t k = 2; k <= 1024; k <<= 1) {
+      if (k > N) break;  // uniform
+      if (k >= (uint32_t)E) {
+        const T want = (i0 & k) ? ~(T)0 : (T)0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) r[e] ^= want ^ flip;
+        flip = want;
+      }
+#pragma unroll
+      for (uint32_t j = k >> 1; j > 0; j >>= 1) bitonic_stage_regs<E>(r, keys, k, j, true, tid, sync);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) r[e] ^= flip;
+    k0 = 2048;
+  }
+  for (uint32_t k = k0; k <= N; k <<= 1)
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      // j is a constant in the in-thread stages, so that r stays in registers
+      if (j >= (uint32_t)E) bitonic_stage_regs<E>(r, keys, k, j, (i0 & k) == 0, tid, sync);
+      else if (j == 1) bitonic_stage_regs<E>(r, keys, k, 1u, (i0 & k) == 0, tid, sync);
+      else if (j == 2) bitonic_stage_regs<E>(r, keys, k, 2u, (i0 & k) == 0, tid, sync);
+      else bitonic_stage_regs<E>(r, keys, k, 4u, (i0 & k) == 0, tid, sync);
+    }
 }
 
 // The register network on keys[0..N), N = E NT: loads each thread's E keys,

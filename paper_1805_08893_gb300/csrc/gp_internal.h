@@ -107,7 +107,9 @@ cudaError_t launch_warp(const DrawArgs& a, const Uniforms& u, int shader, int wa
 int warp_kernel_blocks_per_sm(int shader, int warps_per_block);
 size_t warp_kernel_smem(int shader, int warps_per_block, uint32_t batch_idx);
 
-// Single-draw sort/hash/phash kernel (gp_reuse.cu).
+// Single-draw sort/hash/phash kernel (gp_reuse.cu).  'threads' of the
+// following: the block's, from the context's threads per group.
+int reuse_block_threads(int dedup, uint32_t threads_per_group);
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads);
 // The smaller shared-memory configuration of a static draw (rows for a third
 // of the capacity, a fuller hash table unless the caller chose its size);
