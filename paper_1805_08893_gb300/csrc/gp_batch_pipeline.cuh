@@ -98,15 +98,15 @@ struct PipeBars {
   uint32_t phase0, phase1;
 };
 
-// Runs batches first, first + stride, ... (< nb) of draw 'a' through the
-// pipeline, in the shared memory 'smem' laid out by L (its palette region is
-// not used: 'palette' points to the skinning palette, SH == 1).  Every thread
-// of the block calls it.  Adds the unique vertices and the batches it shaded
+// Runs batches first, first + stride, ... (< nb) of draw 'a' (dyn: dynamic
+// batches, from a.starts) through the pipeline, in the shared memory 'smem' laid
+// out by L (its palette region is not used: 'palette' points to the skinning
+// palette, SH == 1).  Every thread of the block calls it.  Adds the unique vertices and the batches it shaded
 // to inv_total / nbatches (thread 0).  Returns false after a capacity error
 // or a window that did not land (flagged in a.err), with every copy into
 // shared memory drained.  On return the shared memory is free for reuse.
-template <int DEDUP, int SH, bool DYN>
-__device__ __forceinline__ bool pipeline_run(const DrawArgs& a, const Uniforms& u, const float* palette,
+template <int DEDUP, int SH>
+__device__ __forceinline__ bool pipeline_run(const DrawArgs& a, bool dyn, const Uniforms& u, const float* palette,
                                              unsigned char* smem, const BatchLayout& L, PipeBars& pb,
                                              uint32_t first, uint32_t stride, uint32_t nb,
                                              unsigned long long& inv_total, unsigned long long& nbatches) {
@@ -137,7 +137,7 @@ __device__ __forceinline__ bool pipeline_run(const DrawArgs& a, const Uniforms& 
     for (uint32_t s = tid; s < a.hash_slots; s += NT) S.table[s] = kEmpty;
 
   auto batch_range = [&](uint32_t b, uint32_t& t0, uint32_t& t1) {
-    if (DYN) {
+    if (dyn) {
       t0 = __ldg(a.starts + b);
       t1 = __ldg(a.starts + b + 1);
     } else {

@@ -62,6 +62,11 @@ struct Partition {
 // its groups need in a block (at most kFrameSliceBytes to run), 0 if a
 // batch cannot run that way.
 uint32_t frame_capacities(DrawArgs& a, int method, uint32_t shader, uint32_t group);
+// Lays out the work items of a launch over draws[0..n) (num_batches and the
+// capacities set): sets their items, item_begin and run_end, gives the draws of
+// a class common capacities, and fills item_draw (item -> draw).  Returns the
+// number of items.
+uint32_t frame_classes(FrameDraw* draws, uint32_t n, std::vector<uint32_t>& item_draw);
 uint32_t next_pow2(uint32_t x);
 uint32_t log2u(uint32_t x);
 const char* status_name(gp_status s);

@@ -64,6 +64,66 @@ uint32_t frame_capacities(DrawArgs& a, int method, uint32_t shader, uint32_t gro
   }
 }
 
+// Indices per batch from which a hash/phash draw of smaller groups runs by the
+// whole block all the same: shorter batches share a block better in groups than
+// one after another in a pipeline whose producers take 1,280 indices at a time.
+// The 240-draw frame, whose draws of 128 unique vertices have up to 510 indices:
+// 151 us with those in groups, 146 in runs.
+constexpr uint32_t kRunMinIndices = 384;
+
+uint32_t frame_classes(FrameDraw* draws, uint32_t n, std::vector<uint32_t>& item_draw) {
+  // common capacities per class (hash / parallel hash, shader): the largest of its draws', as long as the
+  // run's shared memory holds them
+  struct Class {
+    DrawArgs cap{};
+    uint32_t end = 0;
+  } classes[2][4];
+  std::vector<int8_t> in_class(n, 0);
+  auto class_of = [&](const FrameDraw& D) -> Class& { return classes[D.method == kFramePHash][D.shader]; };
+  for (uint32_t i = 0; i < n; ++i) {
+    FrameDraw& D = draws[i];
+    D.run_end = 0;
+    if ((D.method != kFrameHash && D.method != kFramePHash) || !D.num_batches) continue;
+    if (D.group != kFrameThreads && D.a.max_batch_idx < kRunMinIndices) continue;
+    DrawArgs cap = class_of(D).cap;
+    cap.max_batch_idx = std::max(cap.max_batch_idx, D.a.max_batch_idx);
+    cap.ucap = std::max(cap.ucap, D.a.ucap);
+    cap.hash_slots = std::max(next_pow2(2 * cap.ucap), std::min(next_pow2(4 * cap.ucap), 1024u));
+    cap.hash_bits = log2u(cap.hash_slots);
+    if (cap.hash_slots > 32768u || frame_reuse_bytes((int)D.method, (int)D.shader, cap) > kFrameReuseBytes) continue;
+    class_of(D).cap = cap;
+    in_class[i] = 1;
+  }
+  // the classes' items first, each class's together
+  item_draw.clear();
+  auto place = [&](uint32_t i, uint32_t per_item) {
+    FrameDraw& D = draws[i];
+    D.items = (D.num_batches + per_item - 1) / per_item;
+    D.item_begin = (uint32_t)item_draw.size();
+    item_draw.insert(item_draw.end(), D.items, i);
+  };
+  for (auto& of_method : classes)
+    for (Class& c : of_method) {
+      if (!c.cap.ucap) continue;
+      for (uint32_t i = 0; i < n; ++i) {
+        FrameDraw& D = draws[i];
+        if (!in_class[i] || &class_of(D) != &c) continue;
+        D.a.max_batch_idx = c.cap.max_batch_idx;
+        D.a.ucap = D.a.row_cap = c.cap.ucap;
+        D.a.hash_slots = c.cap.hash_slots;
+        D.a.hash_bits = c.cap.hash_bits;
+        place(i, 1);
+      }
+      c.end = (uint32_t)item_draw.size();
+    }
+  for (uint32_t i = 0; i < n; ++i) {
+    FrameDraw& D = draws[i];
+    if (in_class[i]) D.run_end = class_of(D).end;
+    else place(i, D.method == kFrameNaive ? 1u : (D.method == kFrameWarp ? kFrameThreads / 32 : kFrameThreads / D.group));
+  }
+  return (uint32_t)item_draw.size();
+}
+
 }  // namespace rt
 }  // namespace gp
 
@@ -267,7 +327,6 @@ gp_status frame_create_locked(gp_ctx* c, const gp_draw_desc* draws, uint32_t n, 
   if (n) f->vertex_bytes /= n;
   // batch counts of the dynamic draws (the partitions ran on the stream)
   if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return abort(cuda_fail(c, e, "partition"));
-  uint32_t item = 0;
   for (uint32_t i = 0; i < n; ++i) {
     FrameDraw& D = f->h_draws[i];
     if (D.dynamic) {
@@ -281,17 +340,11 @@ gp_status frame_create_locked(gp_ctx* c, const gp_draw_desc* draws, uint32_t n, 
       }
       D.num_batches = cnt;
     }
-    const uint32_t per_item = D.method == kFrameNaive ? 1u : (D.method == kFrameWarp ? kFrameThreads / 32 : kFrameThreads / D.group);
-    D.items = (D.num_batches + per_item - 1) / per_item;
-    D.item_begin = item;
-    item += D.items;
     f->cfg[i].batches = D.num_batches;
   }
-  f->total_items = item;
+  std::vector<uint32_t> h_item_draw;
+  const uint32_t item = f->total_items = frame_classes(f->h_draws.data(), n, h_item_draw);
   if (item) {
-    std::vector<uint32_t> h_item_draw(item);
-    for (uint32_t i = 0; i < n; ++i)
-      for (uint32_t j = 0; j < f->h_draws[i].items; ++j) h_item_draw[f->h_draws[i].item_begin + j] = i;
     if ((e = cudaMalloc(&f->d_item_draw, sizeof(uint32_t) * item)) != cudaSuccess ||
         (e = cudaMemcpy(f->d_item_draw, h_item_draw.data(), sizeof(uint32_t) * item, cudaMemcpyHostToDevice)) !=
             cudaSuccess)

@@ -128,7 +128,8 @@ int out_floats(int shader);  // K
 // ---- multi-draw frame (gp_frame.cu)
 enum FrameMethod : int { kFrameNaive = 0, kFrameWarp = 1, kFrameSort = 2, kFrameHash = 3, kFramePHash = 4 };
 constexpr uint32_t kFrameThreads = 256;          // threads per block of the frame kernel
-constexpr uint32_t kFrameSliceBytes = 64 * 1024;  // shared memory for the groups of one block
+constexpr uint32_t kFrameSliceBytes = 64 * 1024;  // shared memory for the groups of one block ...
+constexpr uint32_t kFrameReuseBytes = 69 * 1024;  // ... and for a run: three blocks with it fit an SM
 constexpr uint32_t kFrameUniBytes = (sizeof(Uniforms) + 127) / 128 * 128;  // the current draw's uniforms
 
 struct FrameDraw {
@@ -142,6 +143,8 @@ struct FrameDraw {
   uint32_t item_begin;      // first work item of the entry
   uint32_t items;           // work items of the entry
   uint32_t batch_begin;     // first batch (a serving step runs a sub-range of a draw)
+  uint32_t run_end;         // hash/phash entry whose batches go through runs (a batch per item): the item past the
+                            // last one of its class (frame_classes); 0: not
 };
 
 uint32_t frame_slice_bytes(int method, int shader, uint32_t max_idx, uint32_t ucap, uint32_t slots, uint32_t sort_n,
@@ -149,6 +152,8 @@ uint32_t frame_slice_bytes(int method, int shader, uint32_t max_idx, uint32_t uc
 // Shared memory of a sort/hash/phash draw whose group is the whole block
 // (the pipelined path), with the capacities and out_chunk set in 'a'.
 uint32_t frame_pipe_bytes(int method, int shader, const DrawArgs& a);
+// Shared memory of a run of hash/phash batches with the capacities in 'a'.
+uint32_t frame_reuse_bytes(int method, int shader, const DrawArgs& a);
 size_t frame_smem_bytes();
 int frame_blocks_per_sm();
 // item_draw[i]: the entry of draws[] that work item i belongs to.

@@ -299,7 +299,6 @@ bool launch_step(gp_server* s, StepSlot& st) {
   FrameDraw* h_draws = reinterpret_cast<FrameDraw*>(st.h_block);
   Uniforms* h_uni = reinterpret_cast<Uniforms*>(st.h_block + step_align(sizeof(FrameDraw) * kStepMaxEntries));
   std::vector<uint32_t>& item_draw = s->item_scratch;
-  item_draw.clear();
   for (uint64_t rid : s->active) {
     if (batches >= s->cfg.step_max_batches || n >= kStepMaxEntries) break;
     Request& r = s->reqs[rid];
@@ -344,17 +343,13 @@ bool launch_step(gp_server* s, StepSlot& st) {
     h_uni[n] = r.uni;
     D.batch_begin = r.next;
     D.num_batches = take;
-    const uint32_t per = D.method == kFrameNaive ? 1u : (D.method == kFrameWarp ? kFrameThreads / 32 : kFrameThreads / D.group);
-    D.items = (take + per - 1) / per;
-    D.item_begin = items;
-    for (uint32_t j = 0; j < D.items; ++j) item_draw.push_back(n);
-    items += D.items;
     r.next += take;
     batches += take;
     st.parts.push_back({rid, take});
     ++n;
   }
   if (n == 0) return false;
+  items = frame_classes(h_draws, n, item_draw);
   // pack: move the uniforms down behind the n entries, then the item table,
   // the zeroed work counter and record; point the entries at the device copy
   const size_t o_uni = step_align(sizeof(FrameDraw) * n);
