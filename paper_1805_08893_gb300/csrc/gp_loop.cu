@@ -37,6 +37,7 @@ struct LoopArgs {
   const uint32_t* ring_off;
   const uint32_t* ring;
   uint32_t ring_count;
+  uint32_t ring16;                // 1: the ring array is 16-byte aligned
   const uint32_t* vflags;
   const uint32_t* opp;
   float* out;
@@ -48,10 +49,11 @@ struct LoopArgs {
 };
 
 // Position of vertex v; an id out of range (a bad index or adjacency entry)
-// reads as the origin and flags GP_ERR_INDEX_RANGE.
-__device__ __forceinline__ float3 loop_pos(const LoopArgs& a, uint32_t v) {
+// reads as the origin and sets 'bad'.  No side effects: the loads of several
+// positions go out together.
+__device__ __forceinline__ float3 loop_fetch(const LoopArgs& a, uint32_t v, bool& bad) {
   if (v >= a.num_verts) {
-    atomicOr(a.counters + 2, (unsigned long long)EBIT_INDEX_RANGE);
+    bad = true;
     return make_float3(0.f, 0.f, 0.f);
   }
   const unsigned char* row = a.verts + (size_t)v * a.stride;
@@ -63,7 +65,39 @@ __device__ __forceinline__ float3 loop_pos(const LoopArgs& a, uint32_t v) {
   return make_float3(__ldg(p), __ldg(p + 1), __ldg(p + 2));
 }
 
+constexpr uint32_t kLoopStage = 16;  // triangles staged at once by a warp: all 32 cost more cache than they spare stores
+
+__device__ __forceinline__ void loop_flag(const LoopArgs& a, bool bad) {
+  if (bad) atomicOr(a.counters + 2, (unsigned long long)EBIT_INDEX_RANGE);
+}
+
+// The same, flagging GP_ERR_INDEX_RANGE by itself.
+__device__ __forceinline__ float3 loop_pos(const LoopArgs& a, uint32_t v) {
+  bool bad = false;
+  const float3 p = loop_fetch(a, v, bad);
+  loop_flag(a, bad);
+  return p;
+}
+
+// Ring entries k..k + 3 (k < o1, a multiple of 4), of which the caller uses those
+// in [o0, o1) (o1 <= ring_count): one 16-byte load where the array has all four.
+// Rings of unrelated vertices are read side by side, so every load of a warp
+// touches as many lines as it has lanes: two or three loads a ring instead of six
+// (hash, phash and naive: 54 us with it, 56 without, at 500k triangles; warp
+// voting and sort lose 4 us on a mesh whose rings lie in the order of its
+// triangles, and read entry by entry).
+__device__ __forceinline__ uint4 loop_ring4(const LoopArgs& a, uint32_t k, uint32_t o0, uint32_t o1) {
+  if (a.ring16 && a.ring_count - k >= 4) return __ldg(reinterpret_cast<const uint4*>(a.ring + k));
+  uint4 r = make_uint4(0, 0, 0, 0);
+  if (k >= o0) r.x = __ldg(a.ring + k);
+  if (k + 1 >= o0 && o1 - k > 1) r.y = __ldg(a.ring + k + 1);
+  if (k + 2 >= o0 && o1 - k > 2) r.z = __ldg(a.ring + k + 2);
+  if (k + 3 >= o0 && o1 - k > 3) r.w = __ldg(a.ring + k + 3);
+  return r;
+}
+
 // Loop's vertex rule for vertex v at p.
+template <bool WIDE>
 __device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v, float3 p) {
   if (v >= a.num_verts) return p;
   // ring entries past the ring array (inconsistent adjacency) are not read
@@ -78,11 +112,35 @@ __device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v, float
   const uint32_t n = o1 - o0;
   if (n == 0) return p;
   float sx = 0.f, sy = 0.f, sz = 0.f;
-  for (uint32_t k = o0; k < o1; ++k) {
-    const float3 q = loop_pos(a, __ldg(a.ring + k));
-    sx = __fadd_rn(sx, q.x);
-    sy = __fadd_rn(sy, q.y);
-    sz = __fadd_rn(sz, q.z);
+  if (WIDE) {
+    // 4 entries at a time: their positions' loads in flight together, and the next entries' beside them
+    bool bad = false;
+    uint4 ids = loop_ring4(a, o0 & ~3u, o0, o1);
+    for (uint32_t k = o0 & ~3u;; k += 4) {
+      const uint32_t id[4] = {ids.x, ids.y, ids.z, ids.w};
+      const bool more = o1 - k > 4;  // (k + 4 may wrap)
+      if (more) ids = loop_ring4(a, k + 4, o0, o1);
+      float3 q[4];
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i)
+        if (k + i >= o0 && i < o1 - k) q[i] = loop_fetch(a, id[i], bad);
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i)
+        if (k + i >= o0 && i < o1 - k) {
+          sx = __fadd_rn(sx, q[i].x);
+          sy = __fadd_rn(sy, q[i].y);
+          sz = __fadd_rn(sz, q[i].z);
+        }
+      if (!more) break;
+    }
+    loop_flag(a, bad);
+  } else {
+    for (uint32_t k = o0; k < o1; ++k) {
+      const float3 q = loop_pos(a, __ldg(a.ring + k));
+      sx = __fadd_rn(sx, q.x);
+      sy = __fadd_rn(sy, q.y);
+      sz = __fadd_rn(sz, q.z);
+    }
   }
   const float c = __fmaf_rn(0.25f, cosf(6.283185307179586f / (float)n), 0.375f);
   const float beta = __fdiv_rn(__fmaf_rn(-c, c, 0.625f), (float)n);
@@ -92,51 +150,93 @@ __device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v, float
 }
 
 // Loop's edge rule for edge (pa, pb) with opposite vertices pc (this
-// triangle) and d (the neighbour; kEmpty on a boundary).
-__device__ __forceinline__ float3 loop_odd(const LoopArgs& a, float3 pa, float3 pb, float3 pc, uint32_t d) {
-  if (d == kEmpty)
+// triangle) and pd (the neighbour; none on a boundary).
+__device__ __forceinline__ float3 loop_odd(float3 pa, float3 pb, float3 pc, bool boundary, float3 pd) {
+  if (boundary)
     return make_float3(__fmul_rn(0.5f, __fadd_rn(pa.x, pb.x)), __fmul_rn(0.5f, __fadd_rn(pa.y, pb.y)),
                        __fmul_rn(0.5f, __fadd_rn(pa.z, pb.z)));
-  const float3 pd = loop_pos(a, d);
   return make_float3(__fmaf_rn(0.375f, __fadd_rn(pa.x, pb.x), __fmul_rn(0.125f, __fadd_rn(pc.x, pd.x))),
                      __fmaf_rn(0.375f, __fadd_rn(pa.y, pb.y), __fmul_rn(0.125f, __fadd_rn(pc.y, pd.y))),
                      __fmaf_rn(0.375f, __fadd_rn(pa.z, pb.z), __fmul_rn(0.125f, __fadd_rn(pc.z, pd.z))));
 }
 
-// Writes triangle t's four output triangles from its moved vertices E and
-// positions P (corner order).
-__device__ __forceinline__ void loop_emit(const LoopArgs& a, uint32_t t, const float3* E, const float3* P) {
-  float3 M[3];
+// Writes the four output triangles of each of the warp's triangles [t, t + n), a
+// lane's from its moved vertices E and positions P (corner order).  Called by
+// the whole warp.  A lane's 144 bytes go through shared memory ('stage', 9
+// 16-byte words a lane: an odd stride, no bank conflicts), so that the warp
+// writes whole lines; written by the lanes themselves, each store touched 32 of
+// them.  With the rings read 16 bytes at a time: 500k triangles in 55 us, 62.5
+// before.  (STAGED false, warp voting: its rounds end after a few triangles, and
+// the stage's barriers cost it 4 us of 56 on a grid.)
+template <bool STAGED>
+__device__ __forceinline__ void loop_emit(const LoopArgs& a, uint32_t t, uint32_t n, const float3* E, const float3* P,
+                                          float4* stage, uint32_t lane) {
+  float f[36];
+  if (lane < n) {
+    uint32_t d[3];
+    float3 M[3], D[3];
+    bool bad = false;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) M[k] = loop_odd(a, P[k], P[(k + 1) % 3], P[(k + 2) % 3], __ldg(a.opp + 3 * t + k));
-  const float3 c[12] = {E[0], M[0], M[2], E[1], M[1], M[0], E[2], M[2], M[1], M[0], M[1], M[2]};
-  const float f[36] = {c[0].x, c[0].y, c[0].z, c[1].x, c[1].y, c[1].z, c[2].x, c[2].y, c[2].z,
-                       c[3].x, c[3].y, c[3].z, c[4].x, c[4].y, c[4].z, c[5].x, c[5].y, c[5].z,
-                       c[6].x, c[6].y, c[6].z, c[7].x, c[7].y, c[7].z, c[8].x, c[8].y, c[8].z,
-                       c[9].x, c[9].y, c[9].z, c[10].x, c[10].y, c[10].z, c[11].x, c[11].y, c[11].z};
-  float4* o = reinterpret_cast<float4*>(a.out + (size_t)t * 36);
+    for (int k = 0; k < 3; ++k) d[k] = __ldg(a.opp + 3 * (t + lane) + k);
 #pragma unroll
-  for (int w = 0; w < 9; ++w) __stcs(o + w, make_float4(f[4 * w], f[4 * w + 1], f[4 * w + 2], f[4 * w + 3]));
+    for (int k = 0; k < 3; ++k) D[k] = d[k] != kEmpty ? loop_fetch(a, d[k], bad) : make_float3(0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) M[k] = loop_odd(P[k], P[(k + 1) % 3], P[(k + 2) % 3], d[k] == kEmpty, D[k]);
+    loop_flag(a, bad);
+    const float3 c[12] = {E[0], M[0], M[2], E[1], M[1], M[0], E[2], M[2], M[1], M[0], M[1], M[2]};
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      f[3 * k] = c[k].x;
+      f[3 * k + 1] = c[k].y;
+      f[3 * k + 2] = c[k].z;
+    }
+  }
+  if (!STAGED) {
+    float4* o = reinterpret_cast<float4*>(a.out) + (size_t)(t + lane) * 9;
+#pragma unroll
+    for (int w = 0; w < 9; ++w)
+      if (lane < n) __stcs(o + w, make_float4(f[4 * w], f[4 * w + 1], f[4 * w + 2], f[4 * w + 3]));
+    return;
+  }
+#pragma unroll
+  for (uint32_t l0 = 0; l0 < 32; l0 += kLoopStage) {
+    __syncwarp();  // the stage's last readers
+    if (lane - l0 < kLoopStage && lane < n) {
+#pragma unroll
+      for (int w = 0; w < 9; ++w)
+        stage[9 * (lane - l0) + w] = make_float4(f[4 * w], f[4 * w + 1], f[4 * w + 2], f[4 * w + 3]);
+    }
+    __syncwarp();
+    const uint32_t words = l0 < n ? 9 * min(n - l0, kLoopStage) : 0u;
+    float4* o = reinterpret_cast<float4*>(a.out) + (size_t)(t + l0) * 9;
+#pragma unroll
+    for (uint32_t w = lane; w < 9 * kLoopStage; w += 32)
+      if (w < words) __stcs(o + w, stage[w]);
+  }
 }
 
 __global__ void __launch_bounds__(256) loop_naive_kernel(const __grid_constant__ LoopArgs a) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ float4 stage[8 * 9 * kLoopStage];
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, lane = lane_id(), warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     atomicAdd(a.counters + 0, 3ull * min(blockDim.x, a.num_tris - blockIdx.x * blockDim.x));
     atomicAdd(a.counters + 1, 1ull);
   }
-  if (t >= a.num_tris) return;
+  if (t - lane >= a.num_tris) return;
   float3 E[3], P[3];
+  if (t < a.num_tris) {
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const uint32_t v = __ldg(a.idx + 3 * t + k);
-    P[k] = loop_pos(a, v);
-    E[k] = loop_even(a, v, P[k]);
+    for (int k = 0; k < 3; ++k) {
+      const uint32_t v = __ldg(a.idx + 3 * t + k);
+      P[k] = loop_pos(a, v);
+      E[k] = loop_even<true>(a, v, P[k]);
+    }
   }
-  loop_emit(a, t, E, P);
+  loop_emit<true>(a, t - lane, min(32u, a.num_tris - (t - lane)), E, P, stage + warp * 9 * kLoopStage, lane);
 }
 
 // Evaluates the vertex rule of the warp's new ranks into shared memory.
+template <bool WIDE>
 struct LoopEven {
   const LoopArgs& la;
   const uint32_t* uniq;
@@ -147,19 +247,50 @@ struct LoopEven {
     re = min(re, ucap);  // ranks >= ucap (a flagged capacity error) were not stored
     for (uint32_t r = rb + lane; r < re; r += 32) {
       const uint32_t v = uniq[r];
-      const float3 p = loop_pos(la, v), e = loop_even(la, v, p);
+      const float3 p = loop_pos(la, v), e = loop_even<WIDE>(la, v, p);
       esh[3 * r] = e.x; esh[3 * r + 1] = e.y; esh[3 * r + 2] = e.z;
       psh[3 * r] = p.x; psh[3 * r + 1] = p.y; psh[3 * r + 2] = p.z;
     }
   }
 };
 
+// Shared memory of a block.  The warps' stages lie over what the deduplication
+// alone needs: with 7.0 KB a block (64 unique vertices) instead of 8.5 the rest
+// of the SM's 256 KB stays cache for the rings' positions, which neighbouring
+// batches share.
+struct LoopLayout {
+  uint32_t off_table, off_win, off_uniq, off_map, off_even, off_dense, off_misc, total;
+};
+
+__host__ __device__ inline LoopLayout loop_layout(int dedup, uint32_t cap, uint32_t ucap, uint32_t slots,
+                                                  uint32_t sort_n, uint32_t threads) {
+  LoopLayout L;
+  uint32_t o = 0;
+  L.off_table = o; o += dedup == DEDUP_SORT ? sort_n * 8 : slots * 4;
+  L.off_win = o; o += cap * 4;
+  L.off_uniq = o; o += ucap * 4;
+  const uint32_t stages = threads / 32 * kLoopStage * 144;
+  o = o > stages ? o : stages;
+  L.off_even = o; o += ucap * 24;
+  L.off_misc = o; o += 64 * 4;
+  L.off_map = o; o += ((cap + 1) & ~1u) * 2;
+  L.off_dense = o; o += dedup == DEDUP_SORT ? 0u : slots * 2;
+  L.total = o;
+  return L;
+}
+
+// 56 registers: fewer spill, more leave the batches of 64 threads fewer blocks
+// (500k triangles: 55 us; with 64 registers 58, with 48 57).  What bounds it is
+// the L1's line lookups (a gather is one per lane) and the chain of seven
+// dependent loads; a block running consecutive batches one after another for its
+// L1's sake took 62 to 71 us.
 template <int DEDUP>
-__global__ void __launch_bounds__(512) loop_batched_kernel(const __grid_constant__ LoopArgs la,
+__global__ void __maxnreg__(DEDUP == DEDUP_SORT ? 64 : 56) loop_batched_kernel(const __grid_constant__ LoopArgs la,
                                                            const __grid_constant__ DrawArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const uint32_t b = blockIdx.x, tid = threadIdx.x, NT = blockDim.x;
+  const uint32_t tid = threadIdx.x, NT = blockDim.x;
   const uint32_t nb = la.starts ? *la.num_batches_dev : la.num_batches;
+  const uint32_t b = blockIdx.x;
   if (b >= nb) return;
   uint32_t t0, t1;
   if (la.starts) {
@@ -174,26 +305,23 @@ __global__ void __launch_bounds__(512) loop_batched_kernel(const __grid_constant
     if (tid == 0) atomicOr(a.err, EBIT_CAPACITY);
     return;
   }
-  uint32_t* win = reinterpret_cast<uint32_t*>(smem);
-  uint16_t* map = reinterpret_cast<uint16_t*>(win + cap);
-  uint32_t* uniq = reinterpret_cast<uint32_t*>(map + ((cap + 1) & ~1u));
-  float* esh = reinterpret_cast<float*>(uniq + ucap);
+  const LoopLayout L = loop_layout(DEDUP, cap, ucap, a.hash_slots, a.sort_n, NT);
+  uint32_t* win = reinterpret_cast<uint32_t*>(smem + L.off_win);
+  uint32_t* uniq = reinterpret_cast<uint32_t*>(smem + L.off_uniq);
+  uint16_t* map = reinterpret_cast<uint16_t*>(smem + L.off_map);
+  float* esh = reinterpret_cast<float*>(smem + L.off_even);
   float* psh = esh + 3 * ucap;
-  unsigned char* tail = reinterpret_cast<unsigned char*>(psh + 3 * ucap);
-  tail = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tail) + 15) & ~(uintptr_t)15);
+  uint32_t* misc = reinterpret_cast<uint32_t*>(smem + L.off_misc);
   BatchSmem B;
   B.map = map;
   B.uniq = uniq;
   B.vsh = nullptr;
   if (DEDUP == DEDUP_SORT) {
-    B.keys = reinterpret_cast<unsigned long long*>(tail);
-    tail += (size_t)a.sort_n * 8;
+    B.keys = reinterpret_cast<unsigned long long*>(smem + L.off_table);
   } else {
-    B.table = reinterpret_cast<uint32_t*>(tail);
-    B.dense = reinterpret_cast<uint16_t*>(tail + (size_t)a.hash_slots * 4);
-    tail += (size_t)a.hash_slots * 6;
+    B.table = reinterpret_cast<uint32_t*>(smem + L.off_table);
+    B.dense = reinterpret_cast<uint16_t*>(smem + L.off_dense);
   }
-  uint32_t* misc = reinterpret_cast<uint32_t*>(tail);
   B.ucount = misc;
   B.wsum = misc + 8;
   for (uint32_t i = tid; i < n; i += NT) win[i] = __ldg(la.idx + 3 * t0 + i);
@@ -201,10 +329,14 @@ __global__ void __launch_bounds__(512) loop_batched_kernel(const __grid_constant
     for (uint32_t s = tid; s < a.hash_slots; s += NT) B.table[s] = kEmpty;
   if (tid == 0) *B.ucount = 0;
   __syncthreads();
-  dedup<DEDUP, true>(a, B, win, n, tid, NT, BlockSync(), LoopEven{la, uniq, esh, psh, ucap});
+  dedup<DEDUP, true>(a, B, win, n, tid, NT, BlockSync(), LoopEven<DEDUP != DEDUP_SORT>{la, uniq, esh, psh, ucap});
   __syncthreads();
   const uint32_t U = min(*B.ucount, ucap);
-  for (uint32_t j = tid; j < t1 - t0; j += NT) {
+  // the keys, the ids and the window have been read for the last time
+  float4* stage = reinterpret_cast<float4*>(smem) + (tid >> 5) * 9 * kLoopStage;
+  const uint32_t lane = lane_id();
+  for (uint32_t jw = tid - lane; jw < t1 - t0; jw += NT) {  // warp-uniform
+    const uint32_t j = min(jw + lane, t1 - t0 - 1);  // past the batch: computed and not written
     float3 E[3], P[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -214,7 +346,7 @@ __global__ void __launch_bounds__(512) loop_batched_kernel(const __grid_constant
       E[k] = make_float3(esh[3 * r], esh[3 * r + 1], esh[3 * r + 2]);
       P[k] = make_float3(psh[3 * r], psh[3 * r + 1], psh[3 * r + 2]);
     }
-    loop_emit(la, t0 + j, E, P);
+    loop_emit<true>(la, t0 + jw, min(32u, t1 - t0 - jw), E, P, stage, lane);
   }
   if (tid == 0) {
     atomicAdd(la.counters + 0, (unsigned long long)U);
@@ -222,8 +354,10 @@ __global__ void __launch_bounds__(512) loop_batched_kernel(const __grid_constant
   }
 }
 
-// Algorithm 1 per warp: per-warp shared memory held[32] | ids[S] | map[S].
-__host__ __device__ inline uint32_t loop_warp_bytes(uint32_t S) { return 128 + ((S + 3) & ~3u) * 4 + ((S + 15) & ~15u); }
+// Algorithm 1 per warp: per-warp shared memory held[32] | ids[S] | map[S] | stage.
+__host__ __device__ inline uint32_t loop_warp_bytes(uint32_t S) {
+  return 128 + ((S + 3) & ~3u) * 4 + ((S + 15) & ~15u) + kLoopStage * 144;
+}
 
 __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ LoopArgs la, uint32_t S,
                                                         uint32_t nbatches) {
@@ -233,6 +367,7 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
   uint32_t* held = reinterpret_cast<uint32_t*>(wp);
   uint32_t* widx = held + 32;
   unsigned char* map = reinterpret_cast<unsigned char*>(widx + ((S + 3) & ~3u));
+  float4* stage = reinterpret_cast<float4*>(map + ((S + 15) & ~15u));
   unsigned long long inv = 0, nb = 0;
   for (uint32_t b = blockIdx.x * wpb + warp; b < nbatches; b += gridDim.x * wpb) {
     const uint32_t B0 = b * S, n = min(B0 + S, 3 * la.num_tris) - B0;
@@ -252,7 +387,7 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
       float3 E = make_float3(0.f, 0.f, 0.f), P = E;
       if (lane < fill) {
         P = loop_pos(la, held[lane]);
-        E = loop_even(la, held[lane], P);
+        E = loop_even<false>(la, held[lane], P);
       }
       inv += fill;
       const uint32_t tfirst = (B0 + c) / 3;
@@ -266,7 +401,7 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
           Ec[k] = make_float3(__shfl_sync(kFull, E.x, sl), __shfl_sync(kFull, E.y, sl), __shfl_sync(kFull, E.z, sl));
           Pc[k] = make_float3(__shfl_sync(kFull, P.x, sl), __shfl_sync(kFull, P.y, sl), __shfl_sync(kFull, P.z, sl));
         }
-        if (live) loop_emit(la, tfirst + j, Ec, Pc);
+        loop_emit<false>(la, tfirst + p, min(32u, tris - p), Ec, Pc, stage, lane);
       }
       __syncwarp();  // the next round overwrites held/map
       c += 3 * tris;
@@ -277,13 +412,6 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
     atomicAdd(la.counters + 0, inv);
     atomicAdd(la.counters + 1, nb);
   }
-}
-
-size_t loop_batched_smem(int dedup, uint32_t cap, uint32_t ucap, uint32_t slots, uint32_t sort_n) {
-  size_t o = (size_t)cap * 4 + (size_t)((cap + 1) & ~1u) * 2 + (size_t)ucap * 4 + (size_t)ucap * 24;
-  o = (o + 15) & ~(size_t)15;
-  o += dedup == DEDUP_SORT ? (size_t)sort_n * 8 : (size_t)slots * 6;
-  return o + 64 * 4;
 }
 
 }  // namespace gp
@@ -333,6 +461,7 @@ extern "C" gp_status gp_loop_subdivide(const gp_loop_desc* d) {
   la.ring_off = d->d_ring_offsets;
   la.ring = d->d_ring;
   la.ring_count = (uint32_t)std::min<uint64_t>(d->ring_count, 0xFFFFFFFFu);
+  la.ring16 = reinterpret_cast<uintptr_t>(d->d_ring) % 16 == 0 ? 1u : 0u;
   la.vflags = d->d_vertex_flags;
   la.opp = d->d_opposite;
   la.out = d->d_out;
@@ -370,7 +499,7 @@ extern "C" gp_status gp_loop_subdivide(const gp_loop_desc* d) {
     la.num_batches = (T + la.static_tris - 1) / la.static_tris;
     grid = la.num_batches;
   }
-  const size_t smem = loop_batched_smem(dedup, S, ucap, a.hash_slots, a.sort_n);
+  const size_t smem = loop_layout(dedup, S, ucap, a.hash_slots, a.sort_n, threads).total;
   const void* fn = dedup == DEDUP_SORT ? (const void*)loop_batched_kernel<DEDUP_SORT>
                    : dedup == DEDUP_HASH ? (const void*)loop_batched_kernel<DEDUP_HASH>
                                          : (const void*)loop_batched_kernel<DEDUP_PHASH>;
