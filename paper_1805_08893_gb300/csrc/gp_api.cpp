@@ -325,7 +325,7 @@ gp_status check_index_buf(gp_ctx* c, const gp_index_buf* ib) {
 
 // Enqueues one draw (after validation); fills the ticket's counters.
 gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* vb, uint32_t shader,
-                       const Uniforms& u, const gp_out_buf* ob, Ticket& t, DevRec* rec, Partition* pre) {
+                       const Uniforms& u, const gp_out_buf* ob, Ticket& t, DevRec* rec, Partition* pre, bool captured) {
   const gp_config& cfg = c->cfg;
   const uint32_t T = (uint32_t)(ib->num_indices / 3);
   DrawArgs a{};
@@ -444,11 +444,13 @@ gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* v
       smem + (dedup == DEDUP_SORT && threads > 64 ? (size_t)(threads / 128) * 32 * out_floats((int)shader) * 16 : 0);
   if (counted > 227 * 1024)
     return fail(c, GP_ERR_UNSUPPORTED, "batch configuration needs more than 227 KB of shared memory");
-  // a static draw's smaller configuration, where more blocks of it fit an SM
+  // a static draw's smaller configuration, where more blocks of it fit an SM (a captured draw may be replayed beside
+  // the context's other draws, so it does not use their spill buffer)
   DrawArgs small = a;
-  const bool can_shrink = !dyn && c->spill_blocks && reuse_shrink_static(small, cfg.hash_slots != 0);
+  const bool can_shrink = !dyn && !captured && c->spill_blocks && reuse_shrink_static(small, cfg.hash_slots != 0);
   const size_t small_smem = can_shrink ? reuse_smem_bytes(dedup, (int)shader, small, (int)block) : 0;
-  const uint64_t key = (2ull << 56) | ((uint64_t)dedup << 48) | ((uint64_t)dyn << 47) | ((uint64_t)shader << 40) |
+  const uint64_t key = (2ull << 56) | ((uint64_t)dedup << 48) | ((uint64_t)dyn << 47) | ((uint64_t)captured << 46) |
+                       ((uint64_t)shader << 40) |
                        ((uint64_t)threads << 24) | (uint64_t)smem;  // smem < 2^24
   struct Occ {
     int bpsm;
@@ -556,7 +558,7 @@ gp_status submit_locked(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* 
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
   if (cap != cudaStreamCaptureStatusNone) GP_CUDA(c, cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream));
-  s = enqueue_draw(c, ib, vb, shader, u, ob, t, rec, pre);
+  s = enqueue_draw(c, ib, vb, shader, u, ob, t, rec, pre, cap != cudaStreamCaptureStatusNone);
   if (s != GP_OK) {
     put_event(c, t.ev0);
     put_event(c, t.ev1);

@@ -44,3 +44,45 @@ def test_rows_for_a_third(which, variant, S_, threads, shader):
     assert np.array_equal(got.ids, mesh.indices)
     assert np.array_equal(got.out.view(np.uint32), want.out.view(np.uint32))
     assert np.array_equal(got.inv, B.unique_per_batch(mesh.indices, B.static_starts(mesh.num_tris, S_)))
+
+
+def test_captured_draws_replayed_side_by_side():
+    """Two draws of one context, each captured into a graph, replayed on two streams at once: neither may use memory
+    of the other's (every batch holds more unique vertices than a third of its indices)."""
+    import torch
+    import paper_1805_08893_gb300 as gp
+    mesh = MESHES["distinct"]
+    rng = np.random.default_rng(5)
+    big = mg.Mesh(mesh.vertices, np.concatenate([rng.permutation(6000) for _ in range(200)]).astype(np.uint32), mesh.fmt,
+                  "big")
+    uni, _ = uniforms_for(big, S.SHADER_MVP)
+    want = draw_gpu(big, "naive", S.SHADER_MVP, "static", uni, debug=False).out
+    verts = torch.from_numpy(big.vertices).cuda()
+    # the second graph draws the triangles in reverse order
+    idx = [torch.from_numpy(i.view(np.int32).copy()).cuda()
+           for i in (big.indices, np.ascontiguousarray(big.indices.reshape(-1, 3)[::-1]).reshape(-1))]
+    out = [torch.zeros(big.num_tris * 21, device="cuda") for _ in idx]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    ctx = gp.gp_create("hash", stream=streams[0], batch_indices=768)
+    try:
+        graphs = []
+        for i, o in zip(idx, out):
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=streams[0]):
+                gp.gp_submit_drawcall(ctx, i, verts, gp.GP_SHADER_MVP, uni, o)
+            graphs.append(graph)
+        for _ in range(3):
+            for o in out:
+                o.zero_()
+            torch.cuda.synchronize()
+            for graph, stream in zip(graphs, streams):
+                with torch.cuda.stream(stream):
+                    graph.replay()
+            torch.cuda.synchronize()
+            want = want.reshape(big.num_tris, -1)
+            for o, w in zip(out, (want, want[::-1])):
+                assert np.array_equal(o.cpu().numpy().reshape(want.shape).view(np.uint32),
+                                      np.ascontiguousarray(w).view(np.uint32))
+        del graphs
+    finally:
+        gp.gp_destroy(ctx)
