@@ -135,7 +135,7 @@ __device__ __noinline__ uint2 frame_warp(const FrameDraw& D, const Uniforms& u, 
   if (j >= D.num_batches) return make_uint2(0, 0);
   const uint32_t b = D.batch_begin + j;
   unsigned char* wp = slices + warp * WarpSmem<SH>::per_warp_bytes(3u * a.static_batch_tris);
-  WarpState st;
+  WarpState<kWarpAhead> st;
   st.load(a, b, lane);
   const uint32_t n = warp_vote_batch<SH>(a, u, u.palette, b, 0xFFFFFFFFu, wp, lane, st);
   st.settle(lane);  // the slice is used by the next item

@@ -80,19 +80,20 @@ __device__ __forceinline__ void warp_vote_round(const uint32_t* widx, uint32_t n
 }
 
 // A warp's state across the batches it processes: the next batch's indices,
-// read one batch ahead (batches of at most kWarpAhead indices), and whether a
-// bulk store may still read its staging area.
+// read one batch ahead (batches of at most AHEAD indices), and whether a bulk
+// store may still read its staging area.
 constexpr uint32_t kWarpAhead = 96;
 
+template <uint32_t AHEAD>
 struct WarpState {
-  uint32_t ids[kWarpAhead / 32];
+  uint32_t ids[AHEAD / 32];
   bool pending = false;
 
   __device__ __forceinline__ void load(const DrawArgs& a, uint32_t b, uint32_t lane) {
     const uint32_t S = 3u * a.static_batch_tris;
-    if (S > kWarpAhead) return;
+    if (S > AHEAD) return;
 #pragma unroll
-    for (uint32_t q = 0; q < kWarpAhead / 32; ++q) {
+    for (uint32_t q = 0; q < AHEAD / 32; ++q) {
       const uint32_t i = 32 * q + lane;
       const uint64_t at = (uint64_t)b * S + i;
       ids[q] = i < S && at < a.num_idx ? __ldg(a.idx + at) : 0u;
@@ -114,10 +115,10 @@ struct WarpState {
 // A batch of at most 32 triangles that starts on a 16-byte boundary of the
 // output is assembled whole in the staging area, round by round, and leaves in
 // one bulk store; larger ones are written round by round.
-template <int SH>
+template <int SH, uint32_t AHEAD>
 __device__ __forceinline__ uint32_t warp_vote_batch(const DrawArgs& a, const Uniforms& u, const float* palette,
                                                     uint32_t b, uint32_t next, unsigned char* wp, uint32_t lane,
-                                                    WarpState& st) {
+                                                    WarpState<AHEAD>& st) {
   using L = WarpSmem<SH>;
   constexpr int K = L::K;
   constexpr int F = L::F;
@@ -129,9 +130,9 @@ __device__ __forceinline__ uint32_t warp_vote_batch(const DrawArgs& a, const Uni
   const uint32_t B0 = b * S;
   const uint32_t B1 = min(B0 + S, a.num_idx);
   const uint32_t n = B1 - B0;
-  if (S <= kWarpAhead) {
+  if (S <= AHEAD) {
 #pragma unroll
-    for (uint32_t q = 0; q < kWarpAhead / 32; ++q)
+    for (uint32_t q = 0; q < AHEAD / 32; ++q)
       if (32 * q + lane < n) widx[32 * q + lane] = st.ids[q] < a.num_verts ? st.ids[q] : kInvalidId;
     st.load(a, next, lane);
   } else {
