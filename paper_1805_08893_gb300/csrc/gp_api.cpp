@@ -437,11 +437,11 @@ gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* v
     a.sort_pos_bits = (pb < 32 && (uint64_t)a.num_verts + 1 < (1ull << (32 - pb))) ? pb : 0u;
   }
   a.row_cap = a.ucap;
-  const uint32_t block = (uint32_t)reuse_block_threads(dedup, threads);
+  const uint32_t block = (uint32_t)reuse_block_threads(dedup, threads, shader == GP_SHADER_LOAD ? u.steps : 0u);
   size_t smem = reuse_smem_bytes(dedup, (int)shader, a, (int)block);
-  // the limit counts a staging area for each of the threads / 64 warps that sorting's consumers used to be
+  // the limit counts a staging area for each of the threads / 64 warps that sorting's consumers are in a whole block
   const size_t counted =
-      smem + (dedup == DEDUP_SORT && threads > 64 ? (size_t)(threads / 128) * 32 * out_floats((int)shader) * 16 : 0);
+      smem + (dedup == DEDUP_SORT && block != threads && threads > 64 ? (size_t)(threads / 128) * 32 * out_floats((int)shader) * 16 : 0);
   if (counted > 227 * 1024)
     return fail(c, GP_ERR_UNSUPPORTED, "batch configuration needs more than 227 KB of shared memory");
   // a static draw's smaller configuration, where more blocks of it fit an SM (a captured draw may be replayed beside
@@ -656,7 +656,7 @@ gp_status gp_create(const gp_config* cfg_in, gp_ctx** out) {
     a.sort_pos_bits = 1;
     if (reuse_shrink_static(a, cfg.hash_slots != 0)) {
       const int dedup = cfg.variant == GP_SORT ? DEDUP_SORT : DEDUP_HASH;
-      const size_t smem = reuse_smem_bytes(dedup, GP_SHADER_MVP, a, reuse_block_threads(dedup, th));
+      const size_t smem = reuse_smem_bytes(dedup, GP_SHADER_MVP, a, reuse_block_threads(dedup, th, 0));
       const uint32_t blocks = (uint32_t)c->sms * (uint32_t)std::min<size_t>(5, 227 * 1024 / smem);
       void* p = nullptr;
       if (blocks && cudaMalloc(&p, (size_t)blocks * 4 * (a.ucap - a.row_cap) * sizeof(float4)) == cudaSuccess) {

@@ -109,7 +109,7 @@ size_t warp_kernel_smem(int shader, int warps_per_block, uint32_t batch_idx);
 
 // Single-draw sort/hash/phash kernel (gp_reuse.cu).  'threads' of the
 // following: the block's, from the context's threads per group.
-int reuse_block_threads(int dedup, uint32_t threads_per_group);
+int reuse_block_threads(int dedup, uint32_t threads_per_group, uint32_t steps);  // steps: of the load shader, else 0
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads);
 // The smaller shared-memory configuration of a static draw (rows for a third
 // of the capacity, a fuller hash table unless the caller chose its size);

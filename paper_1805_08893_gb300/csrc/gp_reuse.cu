@@ -13,6 +13,7 @@
 namespace gp {
 
 constexpr uint32_t kReuseBarBytes = 64;
+constexpr uint32_t kSortLoadSteps = 640;
 constexpr uint32_t kDynamicRounds = 6;  // rounds of batches per block claimed from the counter
 
 // Batches [0, nstatic) go to the blocks in turn (block i: i, i + grid, ...);
@@ -158,9 +159,12 @@ bool reuse_shrink_static(DrawArgs& a, bool own_slots) {
 // of the work needs (4.5k of a batch's 21k cycles on four warps): five blocks
 // of 192 threads fit an SM where four of 256 did, 25% more sorting warps.
 // 1.09M triangles at the default limits: 67 us against 81 (with the unrolled network).
-int reuse_block_threads(int dedup, uint32_t threads) {
+// A load of many steps is the consumers' chain: then half of the threads consume
+// (7.2M triangles: a load of 4,096 cycles 527 us against 661, of 16,384 1,431
+// against 1,988; with the network as it was, of 1,024 458 against 384).
+int reuse_block_threads(int dedup, uint32_t threads, uint32_t steps) {
   if (threads <= 64) return 64;
-  return (int)(dedup == DEDUP_SORT ? threads / 4 * 3 : threads);
+  return (int)(dedup == DEDUP_SORT && steps <= kSortLoadSteps ? threads / 4 * 3 : threads);
 }
 
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads) {

@@ -56,10 +56,11 @@ __host__ __device__ inline uint32_t reuse_align16(uint32_t x) { return (x + 15u)
 
 // Producer warps of a block of NT threads (at least 64): hash/phash five
 // eighths, rounded down (5 of 8 warps) -- deduplication is the longer chain
-// of dependent shared-memory round trips; sort two thirds (4 of 6, see
-// reuse_block_threads).  The rest are consumers.
+// of dependent shared-memory round trips; sort half of its threads_per_group: of
+// a block of three quarters of them two thirds (4 of 6), of a whole one half (4 of
+// 8; see reuse_block_threads).  The rest are consumers.
 __host__ __device__ inline uint32_t reuse_producer_warps(uint32_t NT, int dedup) {
-  const uint32_t w = NT / 32, p = dedup == DEDUP_SORT ? (2 * w) / 3 : (5 * w) / 8;
+  const uint32_t w = NT / 32, p = dedup != DEDUP_SORT ? (5 * w) / 8 : ((w & (w - 1)) == 0 ? w / 2 : (2 * w) / 3);
   return p < 1 ? 1 : (p >= w ? w - 1 : p);
 }
 // Groups (4 positions) a producer thread inserts per pass, all CAS in flight.

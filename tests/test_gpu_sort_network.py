@@ -33,3 +33,15 @@ def test_sort_sizes(S_, threads, vertices):
     assert np.array_equal(got.ids, mesh.indices)
     assert np.array_equal(got.out.view(np.uint32), want.out.view(np.uint32))
     assert np.array_equal(got.inv, B.unique_per_batch(mesh.indices, B.static_starts(mesh.num_tris, S_)))
+
+
+@pytest.mark.parametrize("S_,threads", [(255, 64), (510, 128), (768, 256), (2046, 512)])
+@pytest.mark.parametrize("steps", [640, 641])  # either side of the line past which half of the threads consume
+def test_sort_load_steps(S_, threads, steps):
+    mesh = mg.grid_mesh(40)
+    uni, _ = uniforms_for(mesh, S.SHADER_LOAD, steps=steps)
+    want = draw_gpu(mesh, "naive", S.SHADER_LOAD, "static", uni)
+    got = draw_gpu(mesh, "sort", S.SHADER_LOAD, "static", uni, batch_indices=S_, threads_per_group=threads)
+    assert got.status == 0
+    assert np.array_equal(got.out.view(np.uint32), want.out.view(np.uint32))
+    assert np.array_equal(got.inv, B.unique_per_batch(mesh.indices, B.static_starts(mesh.num_tris, S_)))
