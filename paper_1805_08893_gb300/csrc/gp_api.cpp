@@ -158,14 +158,17 @@ gp_status fold(gp_ctx* c, uint64_t upto) {
     Ticket t = c->inflight.front();
     c->inflight.pop_front();
     DevRec ext{};
-    if (t.ext_rec) {  // a frame keeps its own record
+    if (t.ext_rec) {  // a frame keeps its own record, and so does a captured draw
       GP_CUDA(c, cudaMemcpyAsync(&c->h_rec[t.slot], t.ext_rec, sizeof(DevRec), cudaMemcpyDeviceToHost, c->aux));
       GP_CUDA(c, cudaStreamSynchronize(c->aux));
       ext = c->h_rec[t.slot];
     }
     const DevRec& r = t.ext_rec ? ext : c->h_rec[t.slot];
     float ms = 0.f;
-    cudaEventElapsedTime(&ms, t.ev0, t.ev1);
+    if (cudaEventElapsedTime(&ms, t.ev0, t.ev1) != cudaSuccess) {  // a captured draw's events have no times
+      ms = 0.f;
+      cudaGetLastError();  // the next launch would report it
+    }
     put_event(c, t.ev0);
     put_event(c, t.ev1);
     const uint64_t inv = t.device_counts ? r.cnt[CNT_INVOCATIONS] : t.host_inv;
@@ -541,6 +544,29 @@ gp_status new_ticket(gp_ctx* c, Ticket& t) {
   return GP_OK;
 }
 
+// A record for a draw that the caller's stream is capturing.  The graph writes
+// it at every replay, long after the draw's ticket is folded, so it lies outside
+// the ring and is given to no other draw while the context lives.
+gp_status captured_record(gp_ctx* c, DevRec** out) {
+  if (c->captured_left == 0) {
+    constexpr uint32_t kBlock = 64;
+    // a thread with a capture under way may allocate and wait in relaxed mode only
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    GP_CUDA(c, cudaThreadExchangeStreamCaptureMode(&mode));
+    void* p = nullptr;
+    cudaError_t e = ctx_malloc(c, &p, sizeof(DevRec) * kBlock);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, sizeof(DevRec) * kBlock, c->aux);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->aux);
+    if (e != cudaSuccess && p) cudaFree(p);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return cuda_fail(c, e, "record of a captured draw");
+    c->captured.push_back(static_cast<DevRec*>(p));
+    c->captured_left = kBlock;
+  }
+  *out = c->captured.back() + --c->captured_left;
+  return GP_OK;
+}
+
 gp_status submit_locked(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* vb, uint32_t shader,
                         const void* uniforms, uint32_t ubytes, const gp_out_buf* ob, uint64_t* out_ticket,
                         Partition* pre) {
@@ -552,22 +578,32 @@ gp_status submit_locked(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* 
   Ticket t;
   s = new_ticket(c, t);
   if (s != GP_OK) return s;
-  DevRec* rec = c->d_rec + t.slot;
-  GP_CUDA(c, cudaEventRecord(t.ev0, c->stream));
-  // the record is empty (gp_create, fold), but a captured draw runs more than once
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
-  if (cap != cudaStreamCaptureStatusNone) GP_CUDA(c, cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream));
-  s = enqueue_draw(c, ib, vb, shader, u, ob, t, rec, pre, cap != cudaStreamCaptureStatusNone);
+  const bool captured = cap != cudaStreamCaptureStatusNone;
+  DevRec* rec = c->d_rec + t.slot;  // empty (gp_create, fold)
+  auto enqueue = [&]() -> gp_status {
+    GP_CUDA(c, cudaEventRecord(t.ev0, c->stream));
+    if (captured) {
+      gp_status r = captured_record(c, &rec);
+      if (r != GP_OK) return r;
+      t.ext_rec = rec;
+      GP_CUDA(c, cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream));  // at every replay
+    }
+    gp_status r = enqueue_draw(c, ib, vb, shader, u, ob, t, rec, pre, captured);
+    if (r != GP_OK) return r;
+    GP_CUDA(c, cudaEventRecord(t.ev1, c->stream));
+    return GP_OK;
+  };
+  s = enqueue();
   if (s != GP_OK) {
     put_event(c, t.ev0);
     put_event(c, t.ev1);
-    // the id and its slot go to the next draw, the record empty whatever has run
-    cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream);
+    // the id and its slot go to the next draw, the record empty whatever has run (a captured draw's is not used again)
+    if (!captured) cudaMemsetAsync(rec, 0, sizeof(DevRec), c->stream);
     c->next_ticket = t.id;
     return s;
   }
-  GP_CUDA(c, cudaEventRecord(t.ev1, c->stream));
   c->inflight.push_back(t);
   if (out_ticket) *out_ticket = t.id;
   return GP_OK;
@@ -687,6 +723,7 @@ gp_status gp_destroy(gp_ctx* c) {
     for (Partition& p : c->host_parts) release_partition(p);
     for (cudaEvent_t e : c->events) cudaEventDestroy(e);
     if (c->d_rec) cudaFree(c->d_rec);
+    for (DevRec* r : c->captured) cudaFree(r);
     if (c->h_rec) cudaFreeHost(c->h_rec);
     if (c->h_idx) cudaFree(c->h_idx);
     if (c->h_vtx) cudaFree(c->h_vtx);

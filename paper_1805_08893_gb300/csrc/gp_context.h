@@ -39,7 +39,7 @@ struct Ticket {
   bool device_counts = false;
   uint64_t out_bytes = 0;
   uint64_t vertex_bytes_per_inv = 0;
-  const DevRec* ext_rec = nullptr;          // a frame's own record instead of the ring slot
+  const DevRec* ext_rec = nullptr;          // a frame's or a captured draw's own record instead of the ring slot
 };
 
 struct Partition {
@@ -83,6 +83,8 @@ struct gp_ctx {
   int sms = 0;
   gp::rt::DevRec* d_rec = nullptr;
   gp::rt::DevRec* h_rec = nullptr;  // pinned mirror
+  std::vector<gp::rt::DevRec*> captured;  // blocks of records of captured draws ...
+  uint32_t captured_left = 0;             // ... and how many of the last block's are unused
   std::deque<gp::rt::Ticket> inflight;
   uint64_t next_ticket = 1;
   std::vector<cudaEvent_t> events;
