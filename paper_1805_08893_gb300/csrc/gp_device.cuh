@@ -261,7 +261,8 @@ __device__ __forceinline__ void bulk_wait_all() {
 }
 
 // Makes this thread's generic-proxy shared-memory writes visible to the
-// async proxy (a following bulk store reads them).
+// async proxy (a following bulk store reads them, or a bulk load writes over
+// them).
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }

@@ -226,6 +226,15 @@ __host__ __device__ inline BatchLayout frame_pipe_layout(int dedup, int shader, 
                       a.sort_n, a.out_chunk);
 }
 
+// Called by the whole block before it starts a pipeline: the slices hold what
+// the items before wrote there with ordinary stores, and the first index window
+// is bulk-copied over it (another proxy, which a barrier alone does not order
+// behind them).
+__device__ __forceinline__ void order_bulk_copies() {
+  fence_proxy_async_smem();
+  __syncthreads();
+}
+
 // Batches [b0, b1) of a sort/hash/phash draw whose groups are the whole
 // block, through the pipeline.  Returns (unique vertices, batches) for
 // thread 0; (~0u, ~0u) on every thread after an aborted run.
@@ -234,6 +243,7 @@ __device__ __noinline__ uint2 frame_pipe(const FrameDraw& D, const Uniforms& u, 
                                          uint32_t b0, uint32_t b1) {
   const BatchLayout L = frame_pipe_layout(DEDUP, SH, D.a);
   unsigned long long inv = 0, nbat = 0;
+  order_bulk_copies();
   if (!pipeline_run<DEDUP, SH>(D.a, D.dynamic != 0, u, u.palette, slices, L, pb, b0, 1u, b1, inv, nbat))
     return make_uint2(~0u, ~0u);
   return make_uint2((uint32_t)inv, (uint32_t)nbat);
@@ -394,6 +404,7 @@ __device__ __noinline__ bool frame_reuse(const FrameDraw& D, RunSource src, unsi
   }
   for (uint32_t s = 4 * threadIdx.x; s < 2 * a.hash_slots; s += 4 * NT)
     *reinterpret_cast<uint4*>(table + s) = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+  order_bulk_copies();
   reuse_batches<DEDUP, SH, false>(a, *src.su, src.su->palette, slices, L, bars, NT, src);
   __syncthreads();
   const bool ok = misc[2] == 0;

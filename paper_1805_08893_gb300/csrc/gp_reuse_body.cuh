@@ -305,6 +305,7 @@ __device__ __forceinline__ void reuse_batches(const DrawArgs& cap, const Uniform
         const uint32_t p0 = max(end, base);
         if (p0 < i0 + n) {  // uniform per batch
           for (uint32_t i = p0 + tid; i < i0 + n; i += NP) win[i - base] = __ldg(a.idx + i);
+          fence_proxy_async_smem();  // in a run, a later draw's window is bulk-copied over these words
           named_sync(kBarProducers, NP);
         }
       }
