@@ -133,10 +133,20 @@ gp_status wait_event(gp_ctx* c, cudaEvent_t e, uint32_t timeout_ms) {
   }
 }
 
+// How bad an error of a draw is: of several folded together the worst is
+// reported (an index out of range is no failure of gp_stats or of a submit that
+// folds earlier draws, the others are).
+int error_rank(gp_status s) {
+  return s == GP_OK ? 0 : s == GP_ERR_INDEX_RANGE ? 1 : s == GP_ERR_UNSUPPORTED ? 2 : 3;
+}
+
 // Folds completed tickets (front of the queue, up to and including 'upto')
 // into the statistics.  Their events must have completed.
 gp_status fold(gp_ctx* c, uint64_t upto) {
   gp_status worst = GP_OK;
+  auto report = [&](gp_status s, const char* msg) {  // last_error stays that of the returned status
+    if (error_rank(s) >= error_rank(worst)) worst = fail(c, s, msg);
+  };
   if (c->inflight.empty() || c->inflight.front().id > upto) return GP_OK;
   // the records of the folded tickets are consecutive ring slots (maybe wrapping)
   {
@@ -152,7 +162,7 @@ gp_status fold(gp_ctx* c, uint64_t upto) {
     GP_CUDA(c, cudaMemsetAsync(c->d_rec + first, 0, sizeof(DevRec) * run1, c->aux));
     if (n > run1) GP_CUDA(c, cudaMemsetAsync(c->d_rec, 0, sizeof(DevRec) * (n - run1), c->aux));
     GP_CUDA(c, cudaStreamSynchronize(c->aux));
-    if (c->h_rec[kRing].err) worst = fail(c, GP_ERR_UNSUPPORTED, "the dynamic partition exceeded a capacity");
+    if (c->h_rec[kRing].err) report(GP_ERR_UNSUPPORTED, "the dynamic partition exceeded a capacity");
   }
   while (!c->inflight.empty() && c->inflight.front().id <= upto) {
     Ticket t = c->inflight.front();
@@ -181,11 +191,9 @@ gp_status fold(gp_ctx* c, uint64_t upto) {
     c->s_bytes += 4 * t.indices + t.vertex_bytes_per_inv * inv + t.out_bytes;
     c->s_busy += ms;
     c->s_lat.push_back(ms);
-    gp_status s = GP_OK;
-    if (r.err & EBIT_TIMEOUT) s = fail(c, GP_ERR_TIMEOUT, "a bounded device wait gave up");
-    else if (r.err & EBIT_CAPACITY) s = fail(c, GP_ERR_UNSUPPORTED, "a batch exceeded a shared-memory capacity");
-    else if (r.err & EBIT_INDEX_RANGE) s = fail(c, GP_ERR_INDEX_RANGE, "index >= num_vertices in a draw");
-    if (worst == GP_OK) worst = s;
+    if (r.err & EBIT_TIMEOUT) report(GP_ERR_TIMEOUT, "a bounded device wait gave up");
+    else if (r.err & EBIT_CAPACITY) report(GP_ERR_UNSUPPORTED, "a batch exceeded a shared-memory capacity");
+    else if (r.err & EBIT_INDEX_RANGE) report(GP_ERR_INDEX_RANGE, "index >= num_vertices in a draw");
   }
   return worst;
 }
