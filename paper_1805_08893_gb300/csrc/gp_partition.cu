@@ -59,20 +59,20 @@ __global__ void __launch_bounds__(1024) partition_segments_kernel(const __grid_c
   uint32_t* misc = smem_w + 3 * slots;  // [0..31], [32..63]: sums of alternate rounds; [64..95]: scan; [96], [97]: cut
   uint32_t* ring = misc + kPartMisc;
   const uint32_t pbits = p.panel_bits, ring_mask = (kPanels << pbits) - 1, ring_words = 3 * (kPanels << pbits);
+  const uint32_t seg = blockIdx.x;
+  const uint32_t seg_begin = seg * p.segment_tris;
+  const uint32_t seg_end = min(seg_begin + p.segment_tris, p.num_tris);
   const uint32_t num_idx = 3 * p.num_tris;
-  // panel k: the triangles from k << pbits, at that triangle modulo the ring; one group each
+  // panel k: the triangles from k << pbits, at that triangle modulo the ring; one group each (empty past the segment)
   auto fetch_panel = [&](uint32_t k) {
     const uint32_t c = 4 * tid;  // at most 4 tid < 3 << pbits words of a panel (NT >= its 16-byte words)
     if (c < 3u << pbits) {
       const uint64_t w = 3ull * (k << pbits) + c;
-      if (w < num_idx)
+      if (w < 3 * seg_end)
         cp_async16_upto(ring + 3 * ((k << pbits) & ring_mask) + c, p.idx + w, 4 * min(4u, num_idx - (uint32_t)w));
     }
     cp_async_commit();
   };
-  const uint32_t seg = blockIdx.x;
-  const uint32_t seg_begin = seg * p.segment_tris;
-  const uint32_t seg_end = min(seg_begin + p.segment_tris, p.num_tris);
   uint32_t panel = seg_begin >> pbits;  // of the scan's position; panels up to panel + 15 are on their way
   for (uint32_t k = 0; k < kPanels; ++k) fetch_panel(panel + k);
   for (uint32_t s = 4 * tid; s < 3 * slots; s += 4 * NT)
@@ -201,22 +201,155 @@ __global__ void __launch_bounds__(1024) partition_segments_kernel(const __grid_c
   if (tid == 0) p.seg_counts[seg] = count;
 }
 
-// Each block adds up the counts of the segments before its own, then its
-// warps copy one segment's starts each into the final array;
-// starts[total] = T.
+// A warp per segment, where there are segments for several waves of blocks
+// (partition_by_warps): slower through one segment, but with less work.  The
+// window is read into the warp's shared memory; 32 triangles are examined per
+// step, one per lane, their ids' smallest positions in the warp's hash table telling
+// which are new, and a scan of their number tells where the batch ends.
+struct PartLayout {
+  uint32_t keys_off, pos_off, per_warp;
+};
+
+__host__ __device__ inline PartLayout part_layout(uint32_t max_tris, uint32_t slots) {
+  PartLayout L;
+  L.keys_off = ((3 * max_tris + 3) & ~3u) * 4;
+  L.pos_off = L.keys_off + slots * 4;
+  L.per_warp = L.pos_off + slots * 4;
+  return L;
+}
+
+__global__ void __launch_bounds__(256) partition_warps_kernel(const __grid_constant__ PartitionArgs p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const PartLayout L = part_layout(p.max_tris, p.table_slots);
+  const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+  const uint32_t seg = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (seg >= p.num_segments) return;  // warp-uniform; no block barrier in this kernel
+  unsigned char* wb = smem + warp * L.per_warp;
+  uint32_t* win = reinterpret_cast<uint32_t*>(wb);
+  uint32_t* keys = reinterpret_cast<uint32_t*>(wb + L.keys_off);
+  uint32_t* pos = reinterpret_cast<uint32_t*>(wb + L.pos_off);
+  const uint32_t mask = p.table_slots - 1;
+
+  const uint32_t seg_begin = seg * p.segment_tris;
+  const uint32_t seg_end = min(seg_begin + p.segment_tris, p.num_tris);
+  uint32_t* out = p.seg_starts + (size_t)seg * p.seg_cap;
+  uint32_t count = 0;
+  uint32_t t = seg_begin;
+  while (t < seg_end) {
+    if (count >= p.seg_cap) {  // cannot happen: seg_cap bounds the batches of a segment
+      if (lane == 0) atomicOr(p.err, EBIT_CAPACITY);
+      break;
+    }
+    if (lane == 0) out[count] = t;
+    ++count;
+    const uint32_t wt = min(p.max_tris, seg_end - t);
+    const uint32_t nidx = 3 * wt;
+    const uint32_t* src = p.idx + 3 * (size_t)t;
+    for (uint32_t i = lane; i < nidx; i += 32) {
+      const uint32_t x = __ldg(src + i);
+      win[i] = x == kEmpty ? kInvalidId : x;
+    }
+    for (uint32_t s = lane; s < p.table_slots; s += 32) {
+      keys[s] = kEmpty;
+      pos[s] = 0xFFFFFFFFu;
+    }
+    __syncwarp();
+    uint32_t nu = 0;    // unique ids of the batch so far
+    uint32_t cut = wt;  // triangles the batch takes
+    for (uint32_t c = 0; c < wt; c += 32) {
+      const uint32_t j = c + lane;
+      const bool valid = j < wt;
+      // the triangle's three ids: insert them (three independent CAS, then
+      // the rare collisions), record their positions (three independent
+      // atomicMin), and count the ids whose smallest position is here
+      uint32_t x[3], h[3], prev[3];
+      if (valid) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          x[k] = win[3 * j + k];
+          h[k] = part_hash(x[k], p.table_bits);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) prev[k] = atomicCAS(&keys[h[k]], kEmpty, x[k]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          for (uint32_t probes = 0; prev[k] != kEmpty && prev[k] != x[k]; ++probes) {
+            if (probes > p.table_slots) {  // cannot happen: the table has room
+              atomicOr(p.err, EBIT_CAPACITY);
+              break;
+            }
+            h[k] = (h[k] + 1) & mask;
+            prev[k] = atomicCAS(&keys[h[k]], kEmpty, x[k]);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) atomicMin(&pos[h[k]], 3 * j + k);
+      }
+      __syncwarp();
+      uint32_t fresh = 0;
+      if (valid) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) fresh += pos[h[k]] == 3 * j + k;
+      }
+      const uint32_t cum = warp_inclusive_scan(fresh);
+      const uint32_t over = __ballot_sync(kFull, valid && nu + cum > p.max_unique);
+      if (over) {
+        cut = max(1u, c + (uint32_t)(__ffs(over) - 1));
+        break;
+      }
+      nu += __shfl_sync(kFull, cum, 31);
+      __syncwarp();
+    }
+    t += cut;
+    __syncwarp();
+  }
+  if (lane == 0) p.seg_counts[seg] = count;
+}
+
+// Many segments: how many batches lie before every kOffsetSegs-th segment, one
+// block going over the counts once.  offsets[k]: before segment k kOffsetSegs.
+constexpr uint32_t kOffsetSegs = 4;  // counts per thread and step
+
+__global__ void __launch_bounds__(1024) partition_offsets_kernel(const __grid_constant__ PartitionArgs p,
+                                                                 uint32_t* offsets) {
+  __shared__ uint32_t warp_sums[33];
+  uint32_t carry = 0;
+  for (uint32_t base = 0; base < p.num_segments; base += kOffsetSegs * blockDim.x) {
+    const uint32_t first = base + kOffsetSegs * threadIdx.x;
+    uint32_t c = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < kOffsetSegs; ++q)
+      if (first + q < p.num_segments) c += min(p.seg_counts[first + q], p.seg_cap);
+    uint32_t total;
+    const uint32_t before = block_exclusive_scan(c, warp_sums, &total);
+    if (first < p.num_segments) offsets[first / kOffsetSegs] = carry + before;
+    carry += total;
+    __syncthreads();
+  }
+}
+
+// Each block adds up the counts of the segments before its own (or has their
+// sum, 'offsets'), then its warps copy one segment's starts each into the final
+// array; starts[total] = T.
 constexpr uint32_t kGatherSegs = 8;
 
-__global__ void __launch_bounds__(256) partition_gather_kernel(const __grid_constant__ PartitionArgs p) {
+__global__ void __launch_bounds__(256) partition_gather_kernel(const __grid_constant__ PartitionArgs p,
+                                                               const uint32_t* offsets) {
   __shared__ uint32_t sums[8];
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
   const uint32_t first = blockIdx.x * kGatherSegs;
   auto count_of = [&](uint32_t s) { return s < p.num_segments ? min(p.seg_counts[s], p.seg_cap) : 0u; };
-  uint32_t c = 0;
-  for (uint32_t s = tid; s < first; s += 256) c += count_of(s);
-  c = __reduce_add_sync(kFull, c);
-  if (lane == 0) sums[warp] = c;
-  __syncthreads();
-  uint32_t o = __reduce_add_sync(kFull, lane < 8 ? sums[lane] : 0u);
+  uint32_t o;
+  if (offsets) {
+    o = offsets[first / kOffsetSegs];
+  } else {
+    uint32_t c = 0;
+    for (uint32_t s = tid; s < first; s += 256) c += count_of(s);
+    c = __reduce_add_sync(kFull, c);
+    if (lane == 0) sums[warp] = c;
+    __syncthreads();
+    o = __reduce_add_sync(kFull, lane < 8 ? sums[lane] : 0u);
+  }
   const uint32_t own = lane < kGatherSegs ? count_of(first + lane) : 0u;  // the block's segments
   o += __reduce_add_sync(kFull, lane < warp ? own : 0u);
   const uint32_t s = first + warp;
@@ -233,36 +366,92 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(const __grid_cons
   }
 }
 
+// Segments above which the batches before each are counted once, by a kernel of its own: below, adding up
+// the counts in every block costs less than another launch.
+constexpr uint32_t kManySegments = 16384;
+
+static uint32_t slots_at_least(uint32_t n, PartitionArgs& p) {
+  p.table_slots = 32;
+  p.table_bits = 5;
+  while (p.table_slots < n) {
+    p.table_slots <<= 1;
+    ++p.table_bits;
+  }
+  return p.table_slots;
+}
+
+// A block's launch shape for a largest window of p.max_tris (3 max_tris <= 4095): one, two or four indices per
+// thread, and a panel's 16-byte words.  Sets the table and the panels; returns the threads.
+static uint32_t block_shape(PartitionArgs& p, uint32_t ipt, size_t* smem) {
+  p.panel_bits = 6;
+  while ((4u << p.panel_bits) < p.max_tris) ++p.panel_bits;
+  slots_at_least(4 * p.max_tris, p);  // a window without a repeated id: at most three quarters full
+  *smem = (3 * (size_t)p.table_slots + kPartMisc + 3 * ((size_t)kPanels << p.panel_bits)) * 4;
+  return std::max((3 * p.max_tris + ipt - 1) / ipt, (3u << p.panel_bits) / 4) + 31 & ~31u;
+}
+
+static cudaError_t launch_warps(PartitionArgs& p, cudaStream_t s) {
+  // a batch inserts at most one step's ids past its limit
+  const size_t per_warp = part_layout(p.max_tris, slots_at_least(2 * (p.max_unique + 96), p)).per_warp;
+  const uint32_t warps = (uint32_t)std::min<size_t>(4, 227u * 1024u / per_warp);
+  const cudaError_t e = cudaFuncSetAttribute(partition_warps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(warps * per_warp));
+  if (e != cudaSuccess) return e;
+  partition_warps_kernel<<<(p.num_segments + warps - 1) / warps, warps * 32, warps * per_warp, s>>>(p);
+  return cudaGetLastError();
+}
+
+// Blocks or warps for the segments.  A block is faster through one segment, warps do less in all: once the blocks
+// come in waves, what counts is the work.  Measured, us, warps first.
+// Long segments: blocks, at the default limits for 500k triangles 167 and 26, 3M of them in random order 238 and 188,
+// 7.2M 187 and 89 (2.9 waves); 1024 / 1365 on 7.2M 436 and 127.  But with many ids past the limit in a window
+// (max_tris >= 4 max_unique) the batch is cut early and most of a block idles: 64 / 341 on 7.2M 247 and 301,
+// 256 / 1365 on 3M in random order (4.8 waves) 404 and 455.
+// Short segments, whose tables and panels are set up for a batch or two: warps from the first full wave on; segments
+// of 256, 500k in random order 31 and 90, a torus 24 and 22; of 1,024, 64 / 64, 3M in random order 101 and 219, a
+// grid 54 and 75.
+// *ipt: one index per thread shortens the chain of a small window (64 triangles: 57 us against 80 at 500k triangles),
+// four issue the fewest instructions (341: 88 us against 139 at 7.2M; 64: 132 against 144).
+static bool partition_by_warps(PartitionArgs p, uint32_t* ipt) {
+  constexpr float kSms = 152.f;
+  *ipt = p.max_tris <= 128 ? 1u : (p.max_tris <= 256 ? 2u : 4u);
+  size_t smem;
+  const uint32_t threads = block_shape(p, *ipt, &smem);
+  const uint32_t resident = std::min(2048u / threads, (uint32_t)(228u * 1024u / (smem + 1024u)));
+  const float waves = (float)p.num_segments / (kSms * (float)resident);
+  if (waves > 1.f) *ipt = 4u;
+  return p.segment_tris < 2048 ? waves >= 1.f : waves >= 1.5f && p.max_tris >= 4 * p.max_unique;
+}
+
+static cudaError_t launch_blocks(PartitionArgs& p, uint32_t ipt, cudaStream_t s) {
+  size_t smem;
+  const uint32_t threads = block_shape(p, ipt, &smem);
+  const void* fn = ipt == 1   ? reinterpret_cast<const void*>(&partition_segments_kernel<1>)
+                   : ipt == 2 ? reinterpret_cast<const void*>(&partition_segments_kernel<2>)
+                              : reinterpret_cast<const void*>(&partition_segments_kernel<4>);
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  if (ipt == 1) partition_segments_kernel<1><<<p.num_segments, threads, smem, s>>>(p);
+  else if (ipt == 2) partition_segments_kernel<2><<<p.num_segments, threads, smem, s>>>(p);
+  else partition_segments_kernel<4><<<p.num_segments, threads, smem, s>>>(p);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_partition(const PartitionArgs& args, cudaStream_t s) {
   PartitionArgs p = args;
+  p.max_tris = std::min(p.max_tris, p.segment_tris);  // a batch ends with its segment
+  uint32_t* offsets = nullptr;
   if (p.num_segments) {
-    // a block holds the largest window: one, two or four indices per thread (3 max_tris <= 4095)
-    // -- one shortens the chain of a small window (64 triangles: 57 us against 80 at 500k triangles), four issue
-    // the fewest instructions on a large one (341: 88 us against 139 at 7.2M; at 500k equal)
-    const uint32_t ipt = p.max_tris <= 128 ? 1u : (p.max_tris <= 256 ? 2u : 4u);
-    p.panel_bits = 6;
-    while ((4u << p.panel_bits) < p.max_tris) ++p.panel_bits;
-    // ... and a panel's 16-byte words
-    const uint32_t threads = std::max((3 * p.max_tris + ipt - 1) / ipt, (3u << p.panel_bits) / 4) + 31 & ~31u;
-    // slots for a window without a repeated id: at most three quarters full
-    p.table_slots = 32;
-    p.table_bits = 5;
-    while (p.table_slots < 4 * p.max_tris) {
-      p.table_slots <<= 1;
-      ++p.table_bits;
-    }
-    const size_t smem = (3 * (size_t)p.table_slots + kPartMisc + 3 * ((size_t)kPanels << p.panel_bits)) * 4;
-    const void* fn = ipt == 1   ? reinterpret_cast<const void*>(&partition_segments_kernel<1>)
-                     : ipt == 2 ? reinterpret_cast<const void*>(&partition_segments_kernel<2>)
-                                : reinterpret_cast<const void*>(&partition_segments_kernel<4>);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    uint32_t ipt;
+    cudaError_t e = partition_by_warps(p, &ipt) ? launch_warps(p, s) : launch_blocks(p, ipt, s);
     if (e != cudaSuccess) return e;
-    if (ipt == 1) partition_segments_kernel<1><<<p.num_segments, threads, smem, s>>>(p);
-    else if (ipt == 2) partition_segments_kernel<2><<<p.num_segments, threads, smem, s>>>(p);
-    else partition_segments_kernel<4><<<p.num_segments, threads, smem, s>>>(p);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (p.num_segments > kManySegments) {
+      offsets = p.seg_counts + p.num_segments;  // as many words again lie there
+      partition_offsets_kernel<<<1, 1024, 0, s>>>(p, offsets);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
   }
-  partition_gather_kernel<<<std::max(1u, (p.num_segments + kGatherSegs - 1) / kGatherSegs), 256, 0, s>>>(p);
+  partition_gather_kernel<<<std::max(1u, (p.num_segments + kGatherSegs - 1) / kGatherSegs), 256, 0, s>>>(p, offsets);
   return cudaGetLastError();
 }
 
