@@ -112,9 +112,7 @@ typedef struct gp_config {
   uint32_t hash_slots;        /* hash table slots, a power of two >= unique capacity and
                                  <= 32768 [the larger of the next power of two >= 2 x
                                  capacity and of min(next power of two >= 4 x capacity,
-                                 1024); static batches of >= 192 indices may run with as
-                                 few as the next power of two >= 4/3 x capacity, where
-                                 that lets more blocks share an SM] */
+                                 1024)] */
   uint32_t segment_tris;      /* dynamic partition: also cut at every multiple of this
                                  many triangles [4096]; GP_SEGMENT_NONE = single scan */
   uint32_t flags;             /* reserved, 0 */
@@ -190,8 +188,9 @@ typedef struct gp_stats_t {
 
 /* Creates a context on cfg->device.  Allocates small device scratch (error
  * word, counters; static sort/hash/phash batches: room for the shaded vertices
- * that a batch holds past a third of its indices, 20 MB at the defaults).  *out is NULL on failure.  GP_ERR_INVALID on a bad
- * configuration (e.g. batch_indices not a multiple of 3, max_unique < 3). */
+ * that a batch holds past its rows in shared memory, 17 MB at the defaults, 23 for
+ * sort).  *out is NULL on failure.  GP_ERR_INVALID on a bad configuration (e.g.
+ * batch_indices not a multiple of 3, max_unique < 3). */
 gp_status gp_create(const gp_config* cfg, gp_ctx** out);
 
 /* Waits for all work of the context, then frees it and its partitions. */

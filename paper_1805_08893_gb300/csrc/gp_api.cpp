@@ -334,6 +334,14 @@ gp_status check_index_buf(gp_ctx* c, const gp_index_buf* ib) {
   return GP_OK;
 }
 
+// Hash table slots of a draw whose batches hold at most ucap unique vertices.
+uint32_t reuse_hash_slots(const gp_config& cfg, uint32_t ucap) {
+  // default: at least 2x the unique capacity, and 4x up to 1024 slots (fewer
+  // collisions, so shorter probe sequences, where the table stays small)
+  const uint32_t slots = cfg.hash_slots ? cfg.hash_slots : std::max(next_pow2(2 * ucap), std::min(next_pow2(4 * ucap), 1024u));
+  return std::max(slots, next_pow2(cfg.threads_per_group));
+}
+
 // Enqueues one draw (after validation); fills the ticket's counters.
 gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* vb, uint32_t shader,
                        const Uniforms& u, const gp_out_buf* ob, Ticket& t, DevRec* rec, Partition* pre, bool captured) {
@@ -435,10 +443,7 @@ gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* v
   }
   if (cfg.hash_slots && cfg.hash_slots < a.ucap)
     return fail(c, GP_ERR_INVALID, "hash_slots must be at least the unique-vertex capacity of a batch");
-  // default: at least 2x the unique capacity, and 4x up to 1024 slots (fewer
-  // collisions, so shorter probe sequences, where the table stays small)
-  a.hash_slots = cfg.hash_slots ? cfg.hash_slots : std::max(next_pow2(2 * a.ucap), std::min(next_pow2(4 * a.ucap), 1024u));
-  a.hash_slots = std::max(a.hash_slots, next_pow2(threads));
+  a.hash_slots = reuse_hash_slots(cfg, a.ucap);
   if (a.hash_slots > 32768u)  // slots are stored in 15 bits
     return fail(c, GP_ERR_UNSUPPORTED, "hash_slots may be at most 32768");
   a.hash_bits = log2u(a.hash_slots);
@@ -455,49 +460,50 @@ gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* v
       smem + (dedup == DEDUP_SORT && block != threads && threads > 64 ? (size_t)(threads / 128) * 32 * out_floats((int)shader) * 16 : 0);
   if (counted > 227 * 1024)
     return fail(c, GP_ERR_UNSUPPORTED, "batch configuration needs more than 227 KB of shared memory");
-  // a static draw's smaller configuration, where more blocks of it fit an SM (a captured draw may be replayed beside
-  // the context's other draws, so it does not use their spill buffer)
-  DrawArgs small = a;
-  const bool can_shrink = !dyn && !captured && c->spill_blocks && reuse_shrink_static(small, cfg.hash_slots != 0);
-  const size_t small_smem = can_shrink ? reuse_smem_bytes(dedup, (int)shader, small, (int)block) : 0;
-  const uint64_t key = (2ull << 56) | ((uint64_t)dedup << 48) | ((uint64_t)dyn << 47) | ((uint64_t)captured << 46) |
-                       ((uint64_t)shader << 40) |
+  const uint64_t key = (2ull << 56) | ((uint64_t)dedup << 48) | ((uint64_t)dyn << 47) | ((uint64_t)shader << 40) |
                        ((uint64_t)threads << 24) | (uint64_t)smem;  // smem < 2^24
-  struct Occ {
-    int bpsm;
-    bool wide, shrink;
-  } occ{};
-  auto it = c->occ.find(key);
-  if (it != c->occ.end()) {
-    occ = Occ{it->second & 0xFF, (it->second & 0x100) != 0, (it->second & 0x200) != 0};
-  } else {
-    occ.bpsm = reuse_blocks_per_sm(dedup, dyn, (int)shader, (int)block, smem, &occ.wide);
-    if (can_shrink && occ.bpsm > 0) {
-      bool wide = false;
-      const int nb = std::min<int>(reuse_blocks_per_sm(dedup, dyn, (int)shader, (int)block, small_smem, &wide),
-                                   (int)(c->spill_blocks / c->sms));
-      if (nb > occ.bpsm) occ = Occ{nb, wide, true};
+  auto blocks_of = [&](ReuseForm form, size_t bytes) {
+    const uint64_t k = key | ((uint64_t)form + 1) << 50;
+    auto it = c->occ.find(k);
+    if (it == c->occ.end()) it = c->occ.emplace(k, reuse_blocks_per_sm(dedup, form, (int)shader, (int)block, bytes)).first;
+    return it->second;
+  };
+  ReuseForm form = dyn ? ReuseForm::kDynamic : ReuseForm::kStatic;
+  int bpsm = blocks_of(form, smem);
+  if (bpsm <= 0) return fail(c, GP_ERR_UNSUPPORTED, "draw kernel cannot be resident with this configuration");
+  // the 80-register kernel where it exists and fits as many blocks
+  if (dyn && blocks_of(ReuseForm::kWide, smem) == bpsm) form = ReuseForm::kWide;
+  // Fewer rows, where the batches need more blocks than are resident with all of them.  Not where the draw's
+  // vertices are so many that its batches hold more than the rows on average, were each vertex in as few of them
+  // as can be; and not in a captured draw, which may be replayed beside the context's other draws and so does not
+  // use their spill buffer.
+  DrawArgs small = a;
+  if (!dyn && !captured && c->d_spill && a.num_batches > (uint64_t)c->sms * bpsm &&
+      reuse_shrink_static(small, dedup, (int)shader, (int)block) &&
+      (uint64_t)a.num_verts * a.ucap <= (uint64_t)a.num_idx * small.row_cap) {
+    const size_t bytes = reuse_smem_bytes(dedup, (int)shader, small, (int)block);
+    const size_t per_sm = (size_t)c->sms * 4 * (a.ucap - small.row_cap) * sizeof(float4);
+    const int nb = std::min<int>(blocks_of(ReuseForm::kSpill, bytes), (int)(c->spill_bytes / per_sm));
+    if (nb > bpsm) {
+      form = ReuseForm::kSpill;
+      bpsm = nb;
+      a = small;
+      a.spill = c->d_spill;
+      smem = bytes;
     }
-    c->occ[key] = occ.bpsm | (occ.wide ? 0x100 : 0) | (occ.shrink ? 0x200 : 0);
   }
-  if (occ.bpsm <= 0) return fail(c, GP_ERR_UNSUPPORTED, "draw kernel cannot be resident with this configuration");
-  if (occ.shrink) {
-    a = small;
-    a.spill = c->d_spill;
-    smem = small_smem;
-  }
-  uint64_t grid = (uint64_t)c->sms * occ.bpsm;
+  uint64_t grid = (uint64_t)c->sms * bpsm;
   if (!dyn) grid = std::min<uint64_t>(grid, a.num_batches);
   if (std::getenv("GP_VERBOSE") && c->logged.insert(key).second)
     std::fprintf(stderr, "[gp] reuse dedup=%d dyn=%d shader=%u threads=%u smem=%zu blocks/SM=%d grid=%llu slots=%u rows=%u regs=%d\n",
-                 dedup, (int)dyn, shader, block, smem, occ.bpsm, (unsigned long long)grid, a.hash_slots, a.row_cap,
-                 occ.wide ? 80 : 64);
+                 dedup, (int)dyn, shader, block, smem, bpsm, (unsigned long long)grid, a.hash_slots, a.row_cap,
+                 form == ReuseForm::kWide ? 80 : 64);
   if (c->test_stall_draws) {  // failure injection: this draw's bounded window wait runs out
     --c->test_stall_draws;
     a.test_stall = 1;
   }
   t.device_counts = true;
-  GP_CUDA(c, launch_reuse(dedup, dyn, occ.wide, a, u, (int)shader, (int)block, (int)std::max<uint64_t>(grid, 1), smem,
+  GP_CUDA(c, launch_reuse(dedup, form, a, u, (int)shader, (int)block, (int)std::max<uint64_t>(grid, 1), smem,
                           c->stream));
   return GP_OK;
 }
@@ -692,23 +698,28 @@ gp_status gp_create(const gp_config* cfg_in, gp_ctx** out) {
     return s;
   }
   if (cfg.variant >= GP_SORT && cfg.variant <= GP_PHASH && cfg.mode == GP_BATCH_STATIC) {
-    // room for the static draws' smaller configuration (without it they run with all their rows in shared memory)
+    // room for the vertices past the rows of static draws' batches (without it they run with a row for each)
     DrawArgs a{};
     a.max_batch_idx = a.ucap = cfg.batch_indices;
-    a.hash_slots = cfg.hash_slots ? cfg.hash_slots : 1u << 15;
+    a.hash_slots = reuse_hash_slots(cfg, a.ucap);
     a.sort_n = next_pow2(a.ucap);
     a.sort_pos_bits = 1;
-    if (reuse_shrink_static(a, cfg.hash_slots != 0)) {
-      const int dedup = cfg.variant == GP_SORT ? DEDUP_SORT : DEDUP_HASH;
-      const size_t smem = reuse_smem_bytes(dedup, GP_SHADER_MVP, a, reuse_block_threads(dedup, th, 0));
-      const uint32_t blocks = (uint32_t)c->sms * (uint32_t)std::min<size_t>(5, 227 * 1024 / smem);
-      void* p = nullptr;
-      if (blocks && cudaMalloc(&p, (size_t)blocks * 4 * (a.ucap - a.row_cap) * sizeof(float4)) == cudaSuccess) {
-        c->d_spill = static_cast<float4*>(p);
-        c->spill_blocks = blocks;
-      } else {
-        cudaGetLastError();
+    const int dedup = cfg.variant == GP_SORT ? DEDUP_SORT : DEDUP_HASH;
+    size_t need = 0;
+    for (uint32_t shader = 0; shader <= GP_SHADER_LOAD; ++shader)
+      for (uint32_t steps : {0u, ~0u}) {
+        DrawArgs small = a;
+        const int block = reuse_block_threads(dedup, th, steps);
+        if (!reuse_shrink_static(small, dedup, (int)shader, block)) continue;
+        const size_t smem = reuse_smem_bytes(dedup, (int)shader, small, block) + 1024;
+        need = std::max(need, (size_t)c->sms * (228 * 1024 / smem) * 4 * (a.ucap - small.row_cap) * sizeof(float4));
       }
+    void* p = nullptr;
+    if (need && cudaMalloc(&p, need) == cudaSuccess) {
+      c->d_spill = static_cast<float4*>(p);
+      c->spill_bytes = need;
+    } else {
+      cudaGetLastError();
     }
   }
   *out = c;

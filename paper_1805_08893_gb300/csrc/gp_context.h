@@ -112,10 +112,10 @@ struct gp_ctx {
   // occupancy cache: key -> blocks per SM
   std::unordered_map<uint64_t, int> occ;
   std::unordered_set<uint64_t> logged;
-  // static sort/hash/phash draws: shaded vertices past the rows of a batch in shared memory (DrawArgs::spill),
-  // for spill_blocks blocks; made by gp_create
+  // static sort/hash/phash draws: shaded vertices past the rows of a batch in shared memory (DrawArgs::spill);
+  // made by gp_create
   float4* d_spill = nullptr;
-  uint32_t spill_blocks = 0;
+  size_t spill_bytes = 0;
   // autotune table (frame draws with GP_AUTO), see gp_frame_api.cpp
   std::vector<gp_autotune_entry> tune;
   // gp_draw_host: copy streams (created on first use), so that uploads, draws

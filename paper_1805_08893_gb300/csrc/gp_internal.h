@@ -111,15 +111,19 @@ size_t warp_kernel_smem(int shader, int warps_per_block, uint32_t batch_idx);
 // following: the block's, from the context's threads per group.
 int reuse_block_threads(int dedup, uint32_t threads_per_group, uint32_t steps);  // steps: of the load shader, else 0
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads);
-// The smaller shared-memory configuration of a static draw (rows for a third
-// of the capacity, a fuller hash table unless the caller chose its size);
-// false: the batch is too small to gain from it.
-bool reuse_shrink_static(DrawArgs& a, bool own_slots);
-// Blocks per SM of the 64-register kernel; *wide: the 80-register kernel
-// exists for this draw and fits as many (launch it instead).
-int reuse_blocks_per_sm(int dedup, bool dynamic, int shader, int threads, size_t smem, bool* wide);
-cudaError_t launch_reuse(int dedup, bool dynamic, bool wide, const DrawArgs& a, const Uniforms& u, int shader,
-                         int threads, int grid, size_t smem, cudaStream_t s);
+// A static draw's configuration with fewer rows (row_cap set), so that more
+// blocks share an SM; false: there is none.
+bool reuse_shrink_static(DrawArgs& a, int dedup, int shader, int threads);
+enum class ReuseForm : int {
+  kDynamic,  // dynamic batches, 64 registers a thread
+  kWide,     // dynamic batches, 80 registers: hash/phash, MVP and envelope shader
+  kStatic,   // static batches, a row for every vertex
+  kSpill,    // static batches, rows for some and the rest in a.spill
+};
+// Blocks of the kernel that fit an SM (0: there is no such kernel, or none fits).
+int reuse_blocks_per_sm(int dedup, ReuseForm form, int shader, int threads, size_t smem);
+cudaError_t launch_reuse(int dedup, ReuseForm form, const DrawArgs& a, const Uniforms& u, int shader, int threads,
+                         int grid, size_t smem, cudaStream_t s);
 
 cudaError_t launch_partition(const PartitionArgs& p, cudaStream_t s);
 

@@ -51,7 +51,7 @@ struct DrawSource {
   }
 };
 
-template <int DEDUP, int SH, bool DYN>
+template <int DEDUP, int SH, bool DYN, bool SPILL>
 __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u) {
   extern __shared__ __align__(128) unsigned char block_smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(block_smem);  // and behind them what reuse_layout lays out
@@ -59,7 +59,7 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
   const uint32_t tid = threadIdx.x, NT = blockDim.x;
   DrawSource<DYN> src(a);
   if (src.first() >= src.end()) return;
-  const ReuseLayout L = reuse_layout(DEDUP, SH, a, NT, DYN ? a.ucap : a.row_cap, true);
+  const ReuseLayout L = reuse_layout(DEDUP, SH, a, NT, SPILL ? a.row_cap : a.ucap, true);
   uint32_t* misc = reinterpret_cast<uint32_t*>(smem + L.off_misc);
   uint32_t* table = reinterpret_cast<uint32_t*>(smem + L.off_scratch);
   float* palette = reinterpret_cast<float*>(smem + L.off_pal);
@@ -72,15 +72,15 @@ __device__ __forceinline__ void reuse_body(const DrawArgs& a, const Uniforms& u)
     for (uint32_t i = tid; i < 768; i += NT) palette[i] = u.palette[i];
   if (DEDUP != DEDUP_SORT)
     for (uint32_t s = tid; s < 2 * a.hash_slots; s += NT) table[s] = kEmpty;
-  reuse_batches<DEDUP, SH, !DYN>(a, u, palette, smem, L, bars, NT, src);
+  reuse_batches<DEDUP, SH, SPILL>(a, u, palette, smem, L, bars, NT, src);
 }
 
 // The kernel at 64 registers a thread (4 blocks of 256 threads fit an SM's
 // registers) ...
-template <int DEDUP, int SH, bool DYN>
+template <int DEDUP, int SH, bool DYN, bool SPILL>
 __global__ void __launch_bounds__(512, 2) reuse_kernel(const __grid_constant__ DrawArgs a,
                                                        const __grid_constant__ Uniforms u) {
-  reuse_body<DEDUP, SH, DYN>(a, u);
+  reuse_body<DEDUP, SH, DYN, SPILL>(a, u);
 }
 
 // ... and at up to 80 (3 blocks of 256 threads), for hash/phash draws over
@@ -90,67 +90,68 @@ __global__ void __launch_bounds__(512, 2) reuse_kernel(const __grid_constant__ D
 template <int DEDUP, int SH>
 __global__ void __maxnreg__(80) reuse_kernel_wide(const __grid_constant__ DrawArgs a,
                                                   const __grid_constant__ Uniforms u) {
-  reuse_body<DEDUP, SH, true>(a, u);
+  reuse_body<DEDUP, SH, true, false>(a, u);
 }
 
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 
-template <int D, bool DYN>
+template <int D, bool DYN, bool SPILL>
 static const void* reuse_fn_sh(int shader) {
   switch (shader) {
-    case 0: return reinterpret_cast<const void*>(&reuse_kernel<D, 0, DYN>);
-    case 1: return reinterpret_cast<const void*>(&reuse_kernel<D, 1, DYN>);
-    case 2: return reinterpret_cast<const void*>(&reuse_kernel<D, 2, DYN>);
-    default: return reinterpret_cast<const void*>(&reuse_kernel<D, 3, DYN>);
+    case 0: return reinterpret_cast<const void*>(&reuse_kernel<D, 0, DYN, SPILL>);
+    case 1: return reinterpret_cast<const void*>(&reuse_kernel<D, 1, DYN, SPILL>);
+    case 2: return reinterpret_cast<const void*>(&reuse_kernel<D, 2, DYN, SPILL>);
+    default: return reinterpret_cast<const void*>(&reuse_kernel<D, 3, DYN, SPILL>);
   }
 }
 
-static const void* reuse_kernel_ptr(int dedup, bool dyn, int shader, bool wide) {
-  if (wide) {  // instantiated for hash/phash, dynamic batches, shaders 0 and 2 only
-    if (dedup == DEDUP_SORT || !dyn || (shader != 0 && shader != 2)) return nullptr;
-    if (dedup == DEDUP_HASH)
-      return shader == 0 ? reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_HASH, 0>)
-                         : reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_HASH, 2>);
-    return shader == 0 ? reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_PHASH, 0>)
-                       : reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_PHASH, 2>);
-  }
-  if (dyn) {
-    switch (dedup) {
-      case DEDUP_SORT: return reuse_fn_sh<DEDUP_SORT, true>(shader);
-      case DEDUP_HASH: return reuse_fn_sh<DEDUP_HASH, true>(shader);
-      default: return reuse_fn_sh<DEDUP_PHASH, true>(shader);
-    }
-  }
+template <bool DYN, bool SPILL>
+static const void* reuse_fn(int dedup, int shader) {
   switch (dedup) {
-    case DEDUP_SORT: return reuse_fn_sh<DEDUP_SORT, false>(shader);
-    case DEDUP_HASH: return reuse_fn_sh<DEDUP_HASH, false>(shader);
-    default: return reuse_fn_sh<DEDUP_PHASH, false>(shader);
+    case DEDUP_SORT: return reuse_fn_sh<DEDUP_SORT, DYN, SPILL>(shader);
+    case DEDUP_HASH: return reuse_fn_sh<DEDUP_HASH, DYN, SPILL>(shader);
+    default: return reuse_fn_sh<DEDUP_PHASH, DYN, SPILL>(shader);
   }
+}
+
+static const void* reuse_kernel_ptr(int dedup, ReuseForm form, int shader) {
+  switch (form) {
+    case ReuseForm::kDynamic: return reuse_fn<true, false>(dedup, shader);
+    case ReuseForm::kStatic: return reuse_fn<false, false>(dedup, shader);
+    case ReuseForm::kSpill: return reuse_fn<false, true>(dedup, shader);
+    default: break;  // kWide: instantiated for hash/phash, shaders 0 and 2 only
+  }
+  if (dedup == DEDUP_SORT || (shader != 0 && shader != 2)) return nullptr;
+  if (dedup == DEDUP_HASH)
+    return shader == 0 ? reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_HASH, 0>)
+                       : reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_HASH, 2>);
+  return shader == 0 ? reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_PHASH, 0>)
+                     : reinterpret_cast<const void*>(&reuse_kernel_wide<DEDUP_PHASH, 2>);
 }
 
 // Static batches have room for S unique vertices, yet a batch of a mesh with
-// locality holds a fifth to a third of S: with rows (and table) for all of
-// them a 768-index batch takes 98 KB of a block (skinning: 151 KB, one block
-// per SM).  Here the rows are for a third, the ones past it are shaded from
-// global memory into 'spill', and the table may be three quarters full.  On a
-// skinned 500k-triangle mesh: 3 blocks per SM, 38 us against 55.
-bool reuse_shrink_static(DrawArgs& a, bool own_slots) {
+// locality holds a fifth to a third of S: with rows for all of them a 768-index
+// batch takes 98 KB of a block (skinning: 151 KB, one block per SM).  Here the rows
+// are as many as let more blocks share an SM, at least two ninths of S (768 indices
+// of a torus: 170 vertices), and the vertices past them are shaded from global
+// memory into 'spill'.  700k triangles, S = 768, hash, us, all rows and these: a
+// skinned torus 70 and 44, in random order 124 and 93; MVP 41 and 35, 68 and 57.
+// (The hash table keeps its size: three quarters full it took up to 2.2 times as
+// long on batches without locality.)  A kernel of its own: in one that never spills
+// the code for it cost 2 to 8%.
+bool reuse_shrink_static(DrawArgs& a, int dedup, int shader, int threads) {
   if (a.ucap < 192) return false;
-  a.row_cap = (a.ucap / 3 + 3) & ~3u;
-  if (!own_slots) {
-    uint32_t slots = 1024, bits = 10;
-    while (slots < a.ucap + a.ucap / 3) {
-      slots <<= 1;
-      ++bits;
-    }
-    if (slots < a.hash_slots) {
-      a.hash_slots = slots;
-      a.hash_bits = bits;
-    }
+  const uint32_t row = 2 * (shader == 1 ? 64u : 32u);  // both slots'
+  const uint32_t fixed = reuse_layout(dedup, shader, a, (uint32_t)threads, 0, true).total + kReuseBarBytes;
+  for (uint32_t n = 65536u / (64u * (uint32_t)threads); n > 1; --n) {  // blocks whose registers fit an SM
+    const uint32_t room = 228u * 1024u / n - 1024u;
+    if (fixed + row * (a.ucap * 2 / 9) > room) continue;
+    a.row_cap = (room - fixed) / row & ~3u;
+    return a.row_cap < a.ucap;
   }
-  return true;
+  return false;
 }
 
 // The kernel splits its block into producer and consumer warps: at least two
@@ -184,16 +185,13 @@ static int blocks_per_sm(const void* fn, int threads, size_t smem) {
   return nb;
 }
 
-int reuse_blocks_per_sm(int dedup, bool dynamic, int shader, int threads, size_t smem, bool* wide) {
-  const int nb = blocks_per_sm(reuse_kernel_ptr(dedup, dynamic, shader, false), threads, smem);
-  // the 80-register kernel where it exists and fits as many blocks per SM
-  *wide = nb > 0 && blocks_per_sm(reuse_kernel_ptr(dedup, dynamic, shader, true), threads, smem) == nb;
-  return nb;
+int reuse_blocks_per_sm(int dedup, ReuseForm form, int shader, int threads, size_t smem) {
+  return blocks_per_sm(reuse_kernel_ptr(dedup, form, shader), threads, smem);
 }
 
-cudaError_t launch_reuse(int dedup, bool dynamic, bool wide, const DrawArgs& a, const Uniforms& u, int shader,
-                         int threads, int grid, size_t smem, cudaStream_t s) {
-  const void* fn = reuse_kernel_ptr(dedup, dynamic, shader, wide);
+cudaError_t launch_reuse(int dedup, ReuseForm form, const DrawArgs& a, const Uniforms& u, int shader, int threads,
+                         int grid, size_t smem, cudaStream_t s) {
+  const void* fn = reuse_kernel_ptr(dedup, form, shader);
   if (fn == nullptr) return cudaErrorInvalidValue;
   void* args[] = {const_cast<DrawArgs*>(&a), const_cast<Uniforms*>(&u)};
   return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, s);
