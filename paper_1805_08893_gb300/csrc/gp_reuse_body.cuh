@@ -480,12 +480,13 @@ __device__ __forceinline__ void reuse_batches(const DrawArgs& cap, const Uniform
           if (lane == 0 && total) r = atomicAdd(counter, total);
           r = __shfl_sync(kFull, r, 0) + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt) +
               8 * __popc(b3 & lt);
-          // With the envelope shader, whose producers wait for the consumers, a
-          // warp's new rows are copied one per lane (a lane holds one new id of
-          // every five positions): fewer instructions for the other role,
-          // 103.8 -> 100.9 us on 2M triangles.  Elsewhere each row starts as
-          // soon as its id is known: 198.6 us against 204.2 on the 7.2M-triangle mesh.
-          constexpr bool kGather = SH == 2;
+          // Parallel hashing with the envelope shader, whose producers wait for the
+          // consumers: a warp's new rows are copied one per lane (a lane holds one new
+          // id of every five positions), fewer instructions for the other role; 2M
+          // triangles 101.3 us, 102.8 copied as below.  Elsewhere each row starts as soon
+          // as its id is known: hash 100.2 us (100.6 gathered), on a grid in batches of 64
+          // triangles 231 (252), MVP on the 7.2M-triangle mesh 198.6 (204.2).
+          constexpr bool kGather = SH == 2 && DEDUP == DEDUP_PHASH;
           uint32_t rw = 0;  // the warp's first rank
           if constexpr (kGather) rw = __shfl_sync(kFull, r, 0);
 #pragma unroll
