@@ -453,7 +453,9 @@ gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* v
     a.sort_pos_bits = (pb < 32 && (uint64_t)a.num_verts + 1 < (1ull << (32 - pb))) ? pb : 0u;
   }
   a.row_cap = a.ucap;
-  const uint32_t block = (uint32_t)reuse_block_threads(dedup, threads, shader == GP_SHADER_LOAD ? u.steps : 0u);
+  const uint32_t block =
+      (uint32_t)reuse_block_threads(dedup, threads, a.max_batch_idx, dyn ? T / cfg.max_tris : a.num_batches,
+                                    shader == GP_SHADER_LOAD ? u.steps : 0u);
   size_t smem = reuse_smem_bytes(dedup, (int)shader, a, (int)block);
   // the limit counts a staging area for each of the threads / 64 warps that sorting's consumers are in a whole block
   const size_t counted =
@@ -707,9 +709,9 @@ gp_status gp_create(const gp_config* cfg_in, gp_ctx** out) {
     const int dedup = cfg.variant == GP_SORT ? DEDUP_SORT : DEDUP_HASH;
     size_t need = 0;
     for (uint32_t shader = 0; shader <= GP_SHADER_LOAD; ++shader)
-      for (uint32_t steps : {0u, ~0u}) {
+      for (uint32_t batches : {0u, ~0u}) {
         DrawArgs small = a;
-        const int block = reuse_block_threads(dedup, th, steps);
+        const int block = reuse_block_threads(dedup, th, a.ucap, batches, 0);
         if (!reuse_shrink_static(small, dedup, (int)shader, block)) continue;
         const size_t smem = reuse_smem_bytes(dedup, (int)shader, small, block) + 1024;
         need = std::max(need, (size_t)c->sms * (228 * 1024 / smem) * 4 * (a.ucap - small.row_cap) * sizeof(float4));

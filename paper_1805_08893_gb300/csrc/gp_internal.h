@@ -109,7 +109,8 @@ size_t warp_kernel_smem(int shader, int warps_per_block, uint32_t batch_idx);
 
 // Single-draw sort/hash/phash kernel (gp_reuse.cu).  'threads' of the
 // following: the block's, from the context's threads per group.
-int reuse_block_threads(int dedup, uint32_t threads_per_group, uint32_t steps);  // steps: of the load shader, else 0
+// batch_idx, batches: a batch's largest size and at least how many there are; steps: of the load shader, else 0.
+int reuse_block_threads(int dedup, uint32_t threads_per_group, uint32_t batch_idx, uint64_t batches, uint32_t steps);
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads);
 // A static draw's configuration with fewer rows (row_cap set), so that more
 // blocks share an SM; false: there is none.

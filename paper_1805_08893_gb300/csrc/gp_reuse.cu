@@ -8,12 +8,13 @@
 // so blocks that run faster take more of them and all finish together.
 // The block's work is reuse_batches (gp_reuse_body.cuh): producer warps
 // deduplicate a batch while consumer warps shade and assemble the one before.
+#include <algorithm>
+
 #include "gp_reuse_body.cuh"
 
 namespace gp {
 
 constexpr uint32_t kReuseBarBytes = 64;
-constexpr uint32_t kSortLoadSteps = 640;
 constexpr uint32_t kDynamicRounds = 6;  // rounds of batches per block claimed from the counter
 
 // Batches [0, nstatic) go to the blocks in turn (block i: i, i + grid, ...);
@@ -155,17 +156,20 @@ bool reuse_shrink_static(DrawArgs& a, int dedup, int shader, int threads) {
 }
 
 // The kernel splits its block into producer and consumer warps: at least two
-// warps.  Sort: half of the threads sort (a 1024-key network then keeps 8 keys
-// per thread in registers) and a quarter consume, which is all that their share
-// of the work needs (4.5k of a batch's 21k cycles on four warps): five blocks
-// of 192 threads fit an SM where four of 256 did, 25% more sorting warps.
-// 1.09M triangles at the default limits: 67 us against 81 (with the unrolled network).
-// A load of many steps is the consumers' chain: then half of the threads consume
-// (7.2M triangles: a load of 4,096 cycles 527 us against 661, of 16,384 1,431
-// against 1,988; with the network as it was, of 1,024 458 against 384).
-int reuse_block_threads(int dedup, uint32_t threads, uint32_t steps) {
+// warps.  Sort: half of the threads sort and half consume.  Batches of no more
+// indices than threads are sorted in a few stages; then a quarter consume, which is
+// enough for a light shader, and five blocks of 192 threads fit an SM where four of
+// 256 do -- if there are batches for them all.  700k triangles, MVP, us: S = 96 197
+// in whole blocks, 172 in these; S = 255 107 and 96; but 20k triangles, S = 255 (235
+// batches) 15.1 and 16.3.  1,024-key batches: no difference on 1.09M triangles with
+// MVP (66), and whole blocks are faster on few triangles (envelope, 20k: 0.79 and
+// 0.94 of what a loop over the network took), on vertices without locality and under
+// loads.  A load of 256 steps leaves these blocks ahead (700k, S = 255: 0.91 and 0.99
+// of the same), one of 1,024 does not (1.18 and 1.00).
+int reuse_block_threads(int dedup, uint32_t threads, uint32_t batch_idx, uint64_t batches, uint32_t steps) {
   if (threads <= 64) return 64;
-  return (int)(dedup == DEDUP_SORT && steps <= kSortLoadSteps ? threads / 4 * 3 : threads);
+  const bool small = dedup == DEDUP_SORT && batch_idx <= std::min(threads, 256u) && batches > 304 && steps <= 256;
+  return (int)(small ? threads / 4 * 3 : threads);
 }
 
 size_t reuse_smem_bytes(int dedup, int shader, const DrawArgs& a, int threads) {

@@ -7,7 +7,8 @@
 // through a two-deep ring of shared-memory slots guarded by mbarriers
 // ("full": deduplicated, rows landed; "empty": assembled, slot free):
 //
-//   producer warps (five eighths of the block; sort: half) deduplicate
+//   producer warps (five eighths of the block; sort: half, or two thirds of a
+//     smaller block, reuse_block_threads) deduplicate
 //     batch j into slot j mod 2: the index window (bulk-copied on an
 //     mbarrier one batch ahead, its triangle range left beside it) is read
 //     from the 16-byte boundary at or below the batch's first index, 4 words
