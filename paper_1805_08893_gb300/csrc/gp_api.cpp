@@ -398,7 +398,7 @@ gp_status enqueue_draw(gp_ctx* c, const gp_index_buf* ib, const gp_vertex_buf* v
     const int wpb = std::max(1u, threads / 32);
     const uint64_t key = (1ull << 40) | ((uint64_t)shader << 32) | (uint64_t)wpb;
     auto it = c->occ.find(key);
-    const int bpsm = it != c->occ.end() ? it->second : (c->occ[key] = warp_kernel_blocks_per_sm((int)shader, wpb));
+    const int bpsm = it != c->occ.end() ? it->second : (c->occ[key] = warp_kernel_blocks_per_sm((int)shader, wpb, S));
     const uint64_t want = ((uint64_t)a.num_batches + wpb - 1) / wpb;
     const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)c->sms * bpsm, want));
     if (std::getenv("GP_VERBOSE") && c->logged.insert(key).second)

@@ -3,15 +3,17 @@
 // per-batch work is warp_vote_batch (gp_warp_body.cuh): a chain of ~10 rounds of
 // votes, scattered row loads and shuffles per three batches, bound by the issue
 // of its instructions and the rows' latency.  1.09M triangles, S = 96: 49 us;
-// written and stored round by round, 56.  At most 80 registers a thread (24
-// warps an SM): at 64 or 48 the spills cost more (60 us), without a limit the
-// kernel takes 140 (66 us).
+// written and stored round by round, 56.  The bound of 256 threads lets the compiler
+// choose 80 registers (24 warps an SM; 48 with the envelope shader): at 64 or 48 the
+// spills cost more (60 us), without it the kernel takes 140 (66 us), and asking for
+// three blocks an SM as well makes it spill more at the same 80 (skinning, 700k
+// triangles, S = 48: 67 us against 53).
 #include "gp_warp_body.cuh"
 
 namespace gp {
 
 template <int SH, uint32_t AHEAD>
-__global__ void __launch_bounds__(256, 3) warp_kernel(const __grid_constant__ DrawArgs a,
+__global__ void __launch_bounds__(256) warp_kernel(const __grid_constant__ DrawArgs a,
                                                    const __grid_constant__ Uniforms u) {
   using L = WarpSmem<SH>;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -56,13 +58,16 @@ size_t warp_kernel_smem(int shader, int warps_per_block, uint32_t batch_idx) {
 
 // Batches over 96 indices: up to 256 are read ahead, in registers that would
 // cost the smaller ones (7.2M triangles: S = 255 in 272 us instead of 337, but
-// S = 96 in 319 instead of 291).
+// S = 96 in 319 instead of 291) and the envelope shader its 48 (2 to 5%).  Larger
+// batches read their indices when they start; the kernel without the registers is
+// the better one for them too (grid, S = 258: 32.7 us against 34.9).
 constexpr uint32_t kWarpFar = 256;
 
 template <int SH>
 static const void* warp_fn(uint32_t batch_idx) {
-  return batch_idx <= kWarpAhead ? reinterpret_cast<const void*>(&warp_kernel<SH, kWarpAhead>)
-                                 : reinterpret_cast<const void*>(&warp_kernel<SH, kWarpFar>);
+  const bool far = batch_idx > kWarpAhead && batch_idx <= kWarpFar && SH != 2;
+  return far ? reinterpret_cast<const void*>(&warp_kernel<SH, kWarpFar>)
+             : reinterpret_cast<const void*>(&warp_kernel<SH, kWarpAhead>);
 }
 
 static const void* warp_kernel_ptr(int shader, uint32_t batch_idx) {
@@ -74,9 +79,9 @@ static const void* warp_kernel_ptr(int shader, uint32_t batch_idx) {
   }
 }
 
-int warp_kernel_blocks_per_sm(int shader, int warps_per_block) {
-  const void* fn = warp_kernel_ptr(shader, 96);
-  const size_t smem = warp_kernel_smem(shader, warps_per_block, 96);
+int warp_kernel_blocks_per_sm(int shader, int warps_per_block, uint32_t batch_idx) {
+  const void* fn = warp_kernel_ptr(shader, batch_idx);
+  const size_t smem = warp_kernel_smem(shader, warps_per_block, batch_idx);
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int nb = 0;

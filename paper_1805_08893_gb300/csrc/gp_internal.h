@@ -104,7 +104,7 @@ cudaError_t launch_multi(const DrawArgs& a, const Uniforms& u, int shader, float
                          cudaStream_t s);
 cudaError_t launch_warp(const DrawArgs& a, const Uniforms& u, int shader, int warps_per_block,
                         int grid, cudaStream_t s);
-int warp_kernel_blocks_per_sm(int shader, int warps_per_block);
+int warp_kernel_blocks_per_sm(int shader, int warps_per_block, uint32_t batch_idx);
 size_t warp_kernel_smem(int shader, int warps_per_block, uint32_t batch_idx);
 
 // Single-draw sort/hash/phash kernel (gp_reuse.cu).  'threads' of the
