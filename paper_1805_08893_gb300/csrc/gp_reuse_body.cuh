@@ -326,9 +326,12 @@ __device__ __forceinline__ void reuse_batches(const DrawArgs& cap, const Uniform
       } else {
         const uint32_t mask = a.hash_slots - 1;
         constexpr int Q = 4 * kGroupsPerPass;  // positions per thread and pass
-        // Parallel hashing's few probes alone: all eight positions together, a slot
-        // per round (7.2M triangles: 203 us, one after another 213).
-        constexpr bool kTogether = DEDUP == DEDUP_PHASH;
+        // Collisions all eight positions together, a slot per round: parallel hashing's
+        // few probes alone (7.2M triangles: 203 us, one after another 213), and hashing
+        // with the envelope shader, whose producers wait for the consumers (2M triangles
+        // of a grid, batches of 64: 218 us and 231, at the tuned limits 100.4 and 100.2).
+        // Hashing otherwise one position after another.
+        constexpr bool kTogether = DEDUP == DEDUP_PHASH || SH == 2;
         for (uint32_t gb = 0; gb < ngroups; gb += kGroupsPerPass * NP) {  // warp-uniform
           // a thread's groups: the lanes of a warp take groups NPW apart, so
           // one CAS instruction meets fewer repeats of the same id
@@ -352,10 +355,10 @@ __device__ __forceinline__ void reuse_batches(const DrawArgs& cap, const Uniform
           // the first probe of every position, issued before any result is used
 #pragma unroll
           for (int q = 0; q < Q; ++q) prev[q] = (act >> q) & 1u ? atomicCAS(&tbl[sl[q]], kEmpty, id[q]) : kEmpty;
-          // collisions (6% of the positions at the tuned limits): a thread's
-          // positions still probing are taken up one after another, a slot at a
-          // time, in one loop -- advancing all eight together takes as many
-          // rounds as the longest chain of the warp, ~90 instructions each
+          // collisions (6% of the positions at the tuned limits).  One after another:
+          // a thread's positions still probing, a slot at a time, in one loop --
+          // advancing all eight together takes as many rounds as the longest chain of
+          // the warp, ~90 instructions each
           uint32_t probing = 0;
 #pragma unroll
           for (int q = 0; q < Q; ++q) {
@@ -364,7 +367,8 @@ __device__ __forceinline__ void reuse_batches(const DrawArgs& cap, const Uniform
             else if (prev[q] != id[q]) probing |= 1u << q;
           }
           if constexpr (kTogether) {
-            for (uint32_t round = 1; probing && round < a.probe_k; ++round) {
+            const uint32_t rounds = DEDUP == DEDUP_PHASH ? a.probe_k : a.hash_slots;
+            for (uint32_t round = 1; probing && round < rounds; ++round) {
 #pragma unroll
               for (int q = 0; q < Q; ++q)
                 if ((probing >> q) & 1u) {
@@ -378,10 +382,14 @@ __device__ __forceinline__ void reuse_batches(const DrawArgs& cap, const Uniform
                   if (prev[q] == kEmpty || prev[q] == id[q]) probing &= ~(1u << q);
                 }
             }
+            if (DEDUP == DEDUP_PHASH) {
 #pragma unroll
-            for (int q = 0; q < Q; ++q)
-              if ((probing >> q) & 1u) sl[q] = (sl[q] + 1) & mask;  // the next slot to probe
-            pend = probing;
+              for (int q = 0; q < Q; ++q)
+                if ((probing >> q) & 1u) sl[q] = (sl[q] + 1) & mask;  // the next slot to probe
+              pend = probing;
+            } else if (probing) {  // table full: cannot happen within capacity
+              atomicOr(a.err, EBIT_CAPACITY);
+            }
           } else {
             for (uint32_t tries = 1; probing;) {
               const uint32_t q = __ffs(probing) - 1;
