@@ -354,10 +354,8 @@ __global__ void __maxnreg__(DEDUP == DEDUP_SORT ? 64 : 56) loop_batched_kernel(c
   }
 }
 
-// Algorithm 1 per warp: per-warp shared memory held[32] | ids[S] | map[S] | stage.
-__host__ __device__ inline uint32_t loop_warp_bytes(uint32_t S) {
-  return 128 + ((S + 3) & ~3u) * 4 + ((S + 15) & ~15u) + kLoopStage * 144;
-}
+// Algorithm 1 per warp: per-warp shared memory held[32] | ids[S] | map[S].
+__host__ __device__ inline uint32_t loop_warp_bytes(uint32_t S) { return 128 + ((S + 3) & ~3u) * 4 + ((S + 15) & ~15u); }
 
 __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ LoopArgs la, uint32_t S,
                                                         uint32_t nbatches) {
@@ -367,7 +365,6 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
   uint32_t* held = reinterpret_cast<uint32_t*>(wp);
   uint32_t* widx = held + 32;
   unsigned char* map = reinterpret_cast<unsigned char*>(widx + ((S + 3) & ~3u));
-  float4* stage = reinterpret_cast<float4*>(map + ((S + 15) & ~15u));
   unsigned long long inv = 0, nb = 0;
   for (uint32_t b = blockIdx.x * wpb + warp; b < nbatches; b += gridDim.x * wpb) {
     const uint32_t B0 = b * S, n = min(B0 + S, 3 * la.num_tris) - B0;
@@ -401,7 +398,7 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
           Ec[k] = make_float3(__shfl_sync(kFull, E.x, sl), __shfl_sync(kFull, E.y, sl), __shfl_sync(kFull, E.z, sl));
           Pc[k] = make_float3(__shfl_sync(kFull, P.x, sl), __shfl_sync(kFull, P.y, sl), __shfl_sync(kFull, P.z, sl));
         }
-        loop_emit<false>(la, tfirst + p, min(32u, tris - p), Ec, Pc, stage, lane);
+        loop_emit<false>(la, tfirst + p, min(32u, tris - p), Ec, Pc, nullptr, lane);
       }
       __syncwarp();  // the next round overwrites held/map
       c += 3 * tris;
