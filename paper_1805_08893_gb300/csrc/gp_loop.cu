@@ -50,14 +50,15 @@ struct LoopArgs {
 
 // Position of vertex v; an id out of range (a bad index or adjacency entry)
 // reads as the origin and sets 'bad'.  No side effects: the loads of several
-// positions go out together.
+// positions go out together.  VEC: in one load where the rows allow it.
+template <bool VEC>
 __device__ __forceinline__ float3 loop_fetch(const LoopArgs& a, uint32_t v, bool& bad) {
   if (v >= a.num_verts) {
     bad = true;
     return make_float3(0.f, 0.f, 0.f);
   }
   const unsigned char* row = a.verts + (size_t)v * a.stride;
-  if (a.vec16) {
+  if (VEC && a.vec16) {
     const float4 x = __ldg(reinterpret_cast<const float4*>(row));
     return make_float3(x.x, x.y, x.z);
   }
@@ -72,9 +73,10 @@ __device__ __forceinline__ void loop_flag(const LoopArgs& a, bool bad) {
 }
 
 // The same, flagging GP_ERR_INDEX_RANGE by itself.
+template <bool VEC>
 __device__ __forceinline__ float3 loop_pos(const LoopArgs& a, uint32_t v) {
   bool bad = false;
-  const float3 p = loop_fetch(a, v, bad);
+  const float3 p = loop_fetch<VEC>(a, v, bad);
   loop_flag(a, bad);
   return p;
 }
@@ -97,14 +99,14 @@ __device__ __forceinline__ uint4 loop_ring4(const LoopArgs& a, uint32_t k, uint3
 }
 
 // Loop's vertex rule for vertex v at p.
-template <bool WIDE>
+template <bool WIDE, bool VEC>
 __device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v, float3 p) {
   if (v >= a.num_verts) return p;
   // ring entries past the ring array (inconsistent adjacency) are not read
   const uint32_t o0 = min(__ldg(a.ring_off + v), a.ring_count);
   const uint32_t o1 = max(o0, min(__ldg(a.ring_off + v + 1), a.ring_count));
   if ((__ldg(a.vflags + v) & 1u) && o1 - o0 >= 2) {
-    const float3 b0 = loop_pos(a, __ldg(a.ring + o0)), b1 = loop_pos(a, __ldg(a.ring + o0 + 1));
+    const float3 b0 = loop_pos<VEC>(a, __ldg(a.ring + o0)), b1 = loop_pos<VEC>(a, __ldg(a.ring + o0 + 1));
     return make_float3(__fmaf_rn(0.75f, p.x, __fmul_rn(0.125f, __fadd_rn(b0.x, b1.x))),
                        __fmaf_rn(0.75f, p.y, __fmul_rn(0.125f, __fadd_rn(b0.y, b1.y))),
                        __fmaf_rn(0.75f, p.z, __fmul_rn(0.125f, __fadd_rn(b0.z, b1.z))));
@@ -123,7 +125,7 @@ __device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v, float
       float3 q[4];
 #pragma unroll
       for (uint32_t i = 0; i < 4; ++i)
-        if (k + i >= o0 && i < o1 - k) q[i] = loop_fetch(a, id[i], bad);
+        if (k + i >= o0 && i < o1 - k) q[i] = loop_fetch<VEC>(a, id[i], bad);
 #pragma unroll
       for (uint32_t i = 0; i < 4; ++i)
         if (k + i >= o0 && i < o1 - k) {
@@ -136,7 +138,7 @@ __device__ __forceinline__ float3 loop_even(const LoopArgs& a, uint32_t v, float
     loop_flag(a, bad);
   } else {
     for (uint32_t k = o0; k < o1; ++k) {
-      const float3 q = loop_pos(a, __ldg(a.ring + k));
+      const float3 q = loop_pos<VEC>(a, __ldg(a.ring + k));
       sx = __fadd_rn(sx, q.x);
       sy = __fadd_rn(sy, q.y);
       sz = __fadd_rn(sz, q.z);
@@ -167,21 +169,32 @@ __device__ __forceinline__ float3 loop_odd(float3 pa, float3 pb, float3 pc, bool
 // writes whole lines; written by the lanes themselves, each store touched 32 of
 // them.  With the rings read 16 bytes at a time: 500k triangles in 55 us, 62.5
 // before.  (STAGED false, warp voting: its rounds end after a few triangles, and
-// the stage's barriers cost it 4 us of 56 on a grid.)
-template <bool STAGED>
+// the stage's barriers cost it 4 us of 56 on a grid; and the lean batched kernels.)
+template <bool STAGED, bool VEC, bool SERIAL>
 __device__ __forceinline__ void loop_emit(const LoopArgs& a, uint32_t t, uint32_t n, const float3* E, const float3* P,
                                           float4* stage, uint32_t lane) {
   float f[36];
   if (lane < n) {
-    uint32_t d[3];
-    float3 M[3], D[3];
+    float3 M[3];
     bool bad = false;
+    if (!SERIAL) {
+      uint32_t d[3];
+      float3 D[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) d[k] = __ldg(a.opp + 3 * (t + lane) + k);
+      for (int k = 0; k < 3; ++k) d[k] = __ldg(a.opp + 3 * (t + lane) + k);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) D[k] = d[k] != kEmpty ? loop_fetch(a, d[k], bad) : make_float3(0.f, 0.f, 0.f);
+      for (int k = 0; k < 3; ++k) D[k] = d[k] != kEmpty ? loop_fetch<VEC>(a, d[k], bad) : make_float3(0.f, 0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) M[k] = loop_odd(P[k], P[(k + 1) % 3], P[(k + 2) % 3], d[k] == kEmpty, D[k]);
+      for (int k = 0; k < 3; ++k) M[k] = loop_odd(P[k], P[(k + 1) % 3], P[(k + 2) % 3], d[k] == kEmpty, D[k]);
+    } else {  // the lean kernels' registers: one edge after another
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const uint32_t d = __ldg(a.opp + 3 * (t + lane) + k);
+        float3 D = make_float3(0.f, 0.f, 0.f);
+        if (d != kEmpty) D = loop_fetch<VEC>(a, d, bad);
+        M[k] = loop_odd(P[k], P[(k + 1) % 3], P[(k + 2) % 3], d == kEmpty, D);
+      }
+    }
     loop_flag(a, bad);
     const float3 c[12] = {E[0], M[0], M[2], E[1], M[1], M[0], E[2], M[2], M[1], M[0], M[1], M[2]};
 #pragma unroll
@@ -228,15 +241,15 @@ __global__ void __launch_bounds__(256) loop_naive_kernel(const __grid_constant__
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const uint32_t v = __ldg(a.idx + 3 * t + k);
-      P[k] = loop_pos(a, v);
-      E[k] = loop_even<true>(a, v, P[k]);
+      P[k] = loop_pos<true>(a, v);
+      E[k] = loop_even<true, true>(a, v, P[k]);
     }
   }
-  loop_emit<true>(a, t - lane, min(32u, a.num_tris - (t - lane)), E, P, stage + warp * 9 * kLoopStage, lane);
+  loop_emit<true, true, false>(a, t - lane, min(32u, a.num_tris - (t - lane)), E, P, stage + warp * 9 * kLoopStage, lane);
 }
 
 // Evaluates the vertex rule of the warp's new ranks into shared memory.
-template <bool WIDE>
+template <bool WIDE, bool VEC>
 struct LoopEven {
   const LoopArgs& la;
   const uint32_t* uniq;
@@ -247,17 +260,17 @@ struct LoopEven {
     re = min(re, ucap);  // ranks >= ucap (a flagged capacity error) were not stored
     for (uint32_t r = rb + lane; r < re; r += 32) {
       const uint32_t v = uniq[r];
-      const float3 p = loop_pos(la, v), e = loop_even<WIDE>(la, v, p);
+      const float3 p = loop_pos<VEC>(la, v), e = loop_even<WIDE, VEC>(la, v, p);
       esh[3 * r] = e.x; esh[3 * r + 1] = e.y; esh[3 * r + 2] = e.z;
       psh[3 * r] = p.x; psh[3 * r + 1] = p.y; psh[3 * r + 2] = p.z;
     }
   }
 };
 
-// Shared memory of a block.  The warps' stages lie over what the deduplication
-// alone needs: with 7.0 KB a block (64 unique vertices) instead of 8.5 the rest
-// of the SM's 256 KB stays cache for the rings' positions, which neighbouring
-// batches share.
+// Shared memory of a block.  The warps' stages ('threads': of those that write
+// staged, 0 for the lean kernels) lie over what the deduplication alone needs: with
+// 7.0 KB a block (64 unique vertices) instead of 8.5 the rest of the SM's 256 KB
+// stays cache for the rings' positions, which neighbouring batches share.
 struct LoopLayout {
   uint32_t off_table, off_win, off_uniq, off_map, off_even, off_dense, off_misc, total;
 };
@@ -269,7 +282,8 @@ __host__ __device__ inline LoopLayout loop_layout(int dedup, uint32_t cap, uint3
   L.off_table = o; o += dedup == DEDUP_SORT ? sort_n * 8 : slots * 4;
   L.off_win = o; o += cap * 4;
   L.off_uniq = o; o += ucap * 4;
-  const uint32_t stages = threads / 32 * kLoopStage * 144;
+  const uint32_t with = (cap / 3 + 31) / 32, warps = threads / 32;  // warps with triangles to write
+  const uint32_t stages = (warps < with ? warps : with) * kLoopStage * 144;
   o = o > stages ? o : stages;
   L.off_even = o; o += ucap * 24;
   L.off_misc = o; o += 64 * 4;
@@ -284,10 +298,16 @@ __host__ __device__ inline LoopLayout loop_layout(int dedup, uint32_t cap, uint3
 // the L1's line lookups (a gather is one per lane) and the chain of seven
 // dependent loads; a block running consecutive batches one after another for its
 // L1's sake took 62 to 71 us.
-template <int DEDUP>
-__global__ void __maxnreg__(DEDUP == DEDUP_SORT ? 64 : 56) loop_batched_kernel(const __grid_constant__ LoopArgs la,
-                                                           const __grid_constant__ DrawArgs a) {
+// LEAN, batches of at most half as many triangles as threads: most warps have
+// nothing to write, and what counts is how many blocks share an SM.  40 registers,
+// triangles written by their lanes, rings read entry by entry and, but for sort,
+// positions word by word (hash, S = 96, 2M triangles of a grid, us: 128 threads 227
+// and, as the others, 321; 256 threads 408 and 660).
+template <int DEDUP, bool LEAN>
+__global__ void __maxnreg__(LEAN ? 40 : DEDUP == DEDUP_SORT ? 64 : 56)
+    loop_batched_kernel(const __grid_constant__ LoopArgs la, const __grid_constant__ DrawArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool kVec = !LEAN || DEDUP == DEDUP_SORT;
   const uint32_t tid = threadIdx.x, NT = blockDim.x;
   const uint32_t nb = la.starts ? *la.num_batches_dev : la.num_batches;
   const uint32_t b = blockIdx.x;
@@ -305,7 +325,7 @@ __global__ void __maxnreg__(DEDUP == DEDUP_SORT ? 64 : 56) loop_batched_kernel(c
     if (tid == 0) atomicOr(a.err, EBIT_CAPACITY);
     return;
   }
-  const LoopLayout L = loop_layout(DEDUP, cap, ucap, a.hash_slots, a.sort_n, NT);
+  const LoopLayout L = loop_layout(DEDUP, cap, ucap, a.hash_slots, a.sort_n, LEAN ? 0 : NT);
   uint32_t* win = reinterpret_cast<uint32_t*>(smem + L.off_win);
   uint32_t* uniq = reinterpret_cast<uint32_t*>(smem + L.off_uniq);
   uint16_t* map = reinterpret_cast<uint16_t*>(smem + L.off_map);
@@ -329,7 +349,8 @@ __global__ void __maxnreg__(DEDUP == DEDUP_SORT ? 64 : 56) loop_batched_kernel(c
     for (uint32_t s = tid; s < a.hash_slots; s += NT) B.table[s] = kEmpty;
   if (tid == 0) *B.ucount = 0;
   __syncthreads();
-  dedup<DEDUP, true>(a, B, win, n, tid, NT, BlockSync(), LoopEven<DEDUP != DEDUP_SORT>{la, uniq, esh, psh, ucap});
+  dedup<DEDUP, true>(a, B, win, n, tid, NT, BlockSync(),
+                    LoopEven<!LEAN && DEDUP != DEDUP_SORT, kVec>{la, uniq, esh, psh, ucap});
   __syncthreads();
   const uint32_t U = min(*B.ucount, ucap);
   // the keys, the ids and the window have been read for the last time
@@ -346,7 +367,7 @@ __global__ void __maxnreg__(DEDUP == DEDUP_SORT ? 64 : 56) loop_batched_kernel(c
       E[k] = make_float3(esh[3 * r], esh[3 * r + 1], esh[3 * r + 2]);
       P[k] = make_float3(psh[3 * r], psh[3 * r + 1], psh[3 * r + 2]);
     }
-    loop_emit<true>(la, t0 + jw, min(32u, t1 - t0 - jw), E, P, stage, lane);
+    loop_emit<!LEAN, kVec, LEAN>(la, t0 + jw, min(32u, t1 - t0 - jw), E, P, stage, lane);
   }
   if (tid == 0) {
     atomicAdd(la.counters + 0, (unsigned long long)U);
@@ -383,8 +404,8 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
       }
       float3 E = make_float3(0.f, 0.f, 0.f), P = E;
       if (lane < fill) {
-        P = loop_pos(la, held[lane]);
-        E = loop_even<false>(la, held[lane], P);
+        P = loop_pos<true>(la, held[lane]);
+        E = loop_even<false, true>(la, held[lane], P);
       }
       inv += fill;
       const uint32_t tfirst = (B0 + c) / 3;
@@ -398,7 +419,7 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
           Ec[k] = make_float3(__shfl_sync(kFull, E.x, sl), __shfl_sync(kFull, E.y, sl), __shfl_sync(kFull, E.z, sl));
           Pc[k] = make_float3(__shfl_sync(kFull, P.x, sl), __shfl_sync(kFull, P.y, sl), __shfl_sync(kFull, P.z, sl));
         }
-        loop_emit<false>(la, tfirst + p, min(32u, tris - p), Ec, Pc, nullptr, lane);
+        loop_emit<false, true, false>(la, tfirst + p, min(32u, tris - p), Ec, Pc, nullptr, lane);
       }
       __syncwarp();  // the next round overwrites held/map
       c += 3 * tris;
@@ -416,6 +437,15 @@ __global__ void __launch_bounds__(256) loop_warp_kernel(const __grid_constant__ 
 using namespace gp;
 
 namespace {
+template <bool LEAN>
+const void* loop_fn(int dedup) {
+  switch (dedup) {
+    case DEDUP_SORT: return reinterpret_cast<const void*>(&loop_batched_kernel<DEDUP_SORT, LEAN>);
+    case DEDUP_HASH: return reinterpret_cast<const void*>(&loop_batched_kernel<DEDUP_HASH, LEAN>);
+    default: return reinterpret_cast<const void*>(&loop_batched_kernel<DEDUP_PHASH, LEAN>);
+  }
+}
+
 uint32_t loop_pow2(uint32_t x) {
   uint32_t p = 1;
   while (p < x) p <<= 1;
@@ -496,14 +526,11 @@ extern "C" gp_status gp_loop_subdivide(const gp_loop_desc* d) {
     la.num_batches = (T + la.static_tris - 1) / la.static_tris;
     grid = la.num_batches;
   }
-  const size_t smem = loop_layout(dedup, S, ucap, a.hash_slots, a.sort_n, threads).total;
-  const void* fn = dedup == DEDUP_SORT ? (const void*)loop_batched_kernel<DEDUP_SORT>
-                   : dedup == DEDUP_HASH ? (const void*)loop_batched_kernel<DEDUP_HASH>
-                                         : (const void*)loop_batched_kernel<DEDUP_PHASH>;
+  const bool lean = threads >= 2 * (S / 3);  // see loop_batched_kernel
+  const size_t smem = loop_layout(dedup, S, ucap, a.hash_slots, a.sort_n, lean ? 0 : threads).total;
+  const void* fn = lean ? loop_fn<true>(dedup) : loop_fn<false>(dedup);
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return GP_ERR_UNSUPPORTED;
-  if (dedup == DEDUP_SORT) loop_batched_kernel<DEDUP_SORT><<<grid, threads, smem, s>>>(la, a);
-  else if (dedup == DEDUP_HASH) loop_batched_kernel<DEDUP_HASH><<<grid, threads, smem, s>>>(la, a);
-  else loop_batched_kernel<DEDUP_PHASH><<<grid, threads, smem, s>>>(la, a);
-  return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;
+  void* args[] = {&la, &a};
+  return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, s) == cudaSuccess ? GP_OK : GP_ERR_CUDA;
 }
