@@ -30,7 +30,7 @@
 // nothing stops the scan, and nearest first its reads share no cache lines: a
 // million agents on an 8192 x 8192 field, one cell in 500 active, took 6,570 us a
 // step against 1,400 row by row; an agent with an empty cell beside it goes row by
-// row (1,500, the bounds included).
+// row (1,430, the bounds included).
 #include <algorithm>
 #include <mutex>
 #include <utility>
@@ -516,7 +516,8 @@ extern "C" gp_status gp_random_walk(const gp_walk_desc* d) {
       wa.bound = bound;
     }
   }
-  for (uint32_t k = 0; k < d->steps; ++k) {
+  gp_status queued = GP_OK;
+  for (uint32_t k = 0; k < d->steps && queued == GP_OK; ++k) {
     wa.step = d->first_step + k;
     wa.pin = (k & 1) ? d->d_scratch : d->d_pos;
     wa.pout = (k & 1) ? d->d_pos : d->d_scratch;
@@ -530,10 +531,12 @@ extern "C" gp_status gp_random_walk(const gp_walk_desc* d) {
       else if (dedup == DEDUP_HASH) walk_batched_kernel<DEDUP_HASH><<<grid, threads, smem, s>>>(wa, a);
       else walk_batched_kernel<DEDUP_PHASH><<<grid, threads, smem, s>>>(wa, a);
     }
-    if (cudaGetLastError() != cudaSuccess) return GP_ERR_CUDA;
+    if (cudaGetLastError() != cudaSuccess) queued = GP_ERR_CUDA;
   }
-  if (wa.bound && cudaEventRecord(bound_done, s) != cudaSuccess) return GP_ERR_CUDA;
+  // behind whatever reads the table, also when a launch failed: its next user waits for that
+  if (wa.bound && cudaEventRecord(bound_done, s) != cudaSuccess) queued = GP_ERR_CUDA;
   if (slot_use.owns_lock()) slot_use.unlock();
+  if (queued != GP_OK) return queued;
   if (d->steps & 1) {  // the last step wrote the scratch buffer
     if (cudaMemcpyAsync(d->d_pos, d->d_scratch, (size_t)d->num_agents * 4, cudaMemcpyDeviceToDevice, s) !=
         cudaSuccess)
