@@ -385,14 +385,17 @@ static uint32_t slots_at_least(uint32_t n, PartitionArgs& p) {
 static uint32_t block_shape(PartitionArgs& p, uint32_t ipt, size_t* smem) {
   p.panel_bits = 6;
   while ((4u << p.panel_bits) < p.max_tris) ++p.panel_bits;
-  slots_at_least(4 * p.max_tris, p);  // a window without a repeated id: at most three quarters full
+  // a window without a repeated id fills at most five eighths (three quarters, as windows of a power of two did
+  // with 4 slots a triangle, probe far: 3M triangles in random order, windows of 1,024: 556 us against 228)
+  slots_at_least(24 * p.max_tris / 5, p);
   *smem = (3 * (size_t)p.table_slots + kPartMisc + 3 * ((size_t)kPanels << p.panel_bits)) * 4;
   return std::max((3 * p.max_tris + ipt - 1) / ipt, (3u << p.panel_bits) / 4) + 31 & ~31u;
 }
 
 static cudaError_t launch_warps(PartitionArgs& p, cudaStream_t s) {
-  // a batch inserts at most one step's ids past its limit
-  const size_t per_warp = part_layout(p.max_tris, slots_at_least(2 * (p.max_unique + 96), p)).per_warp;
+  // a batch inserts at most one step's ids past its limit, and no more than its window's
+  const uint32_t ids = std::min(p.max_unique + 96, 3 * p.max_tris);
+  const size_t per_warp = part_layout(p.max_tris, slots_at_least(2 * ids, p)).per_warp;
   const uint32_t warps = (uint32_t)std::min<size_t>(4, 227u * 1024u / per_warp);
   const cudaError_t e = cudaFuncSetAttribute(partition_warps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(warps * per_warp));
@@ -408,8 +411,10 @@ static cudaError_t launch_warps(PartitionArgs& p, cudaStream_t s) {
 // (max_tris >= 4 max_unique) the batch is cut early and most of a block idles: 64 / 341 on 7.2M 247 and 301,
 // 256 / 1365 on 3M in random order (4.8 waves) 404 and 455.
 // Short segments, whose tables and panels are set up for a batch or two: warps from the first full wave on; segments
-// of 256, 500k in random order 31 and 90, a torus 24 and 22; of 1,024, 64 / 64, 3M in random order 101 and 219, a
-// grid 54 and 75.
+// of 256, 500k in random order 31 and 90, a torus 24 and 22; of 1,024, 64 / 64, 3M in random order 102 and 197, a
+// grid 54 and 68.  But blocks for large windows that are seldom cut (max_tris <= 1.5 max_unique; segments of 1,024,
+// 7.2M, 256 / 341: 157 and 103, 1024 / 1365 397 and 158) or never (3 max_tris <= max_unique; segments of 256, 3M in
+// random order, 1024 / 341: 166 and 91).
 // *ipt: one index per thread shortens the chain of a small window (64 triangles: 57 us against 80 at 500k triangles),
 // four issue the fewest instructions (341: 88 us against 139 at 7.2M; 64: 132 against 144).
 static bool partition_by_warps(PartitionArgs p, uint32_t* ipt) {
@@ -420,7 +425,10 @@ static bool partition_by_warps(PartitionArgs p, uint32_t* ipt) {
   const uint32_t resident = std::min(2048u / threads, (uint32_t)(228u * 1024u / (smem + 1024u)));
   const float waves = (float)p.num_segments / (kSms * (float)resident);
   if (waves > 1.f) *ipt = 4u;
-  return p.segment_tris < 2048 ? waves >= 1.f : waves >= 1.5f && p.max_tris >= 4 * p.max_unique;
+  if (p.segment_tris >= 2048) return waves >= 1.5f && p.max_tris >= 4 * p.max_unique;
+  const bool never = 3 * p.max_tris <= p.max_unique, seldom = 2 * p.max_tris <= 3 * p.max_unique;
+  if (p.max_tris >= 256 && (never || (seldom && p.segment_tris >= 1024))) return false;
+  return waves >= 1.f;
 }
 
 static cudaError_t launch_blocks(PartitionArgs& p, uint32_t ipt, cudaStream_t s) {

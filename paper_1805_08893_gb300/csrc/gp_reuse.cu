@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(512, 2) reuse_kernel(const __grid_constant__ D
 // ... and at up to 80 (3 blocks of 256 threads), for hash/phash draws over
 // dynamic batches with the MVP or envelope shader: where shared memory already
 // holds the block to 3 per SM, the extra registers cost no occupancy and spare
-// the compiler's register-limited scheduling (launch_reuse picks it only then).
+// the compiler's register-limited scheduling (draws take it only then).
 template <int DEDUP, int SH>
 __global__ void __maxnreg__(80) reuse_kernel_wide(const __grid_constant__ DrawArgs a,
                                                   const __grid_constant__ Uniforms u) {

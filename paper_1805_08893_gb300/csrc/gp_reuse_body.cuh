@@ -67,8 +67,8 @@ __host__ __device__ inline uint32_t reuse_producer_warps(uint32_t NT, int dedup)
 // Groups (4 positions) a producer thread inserts per pass, all CAS in flight.
 constexpr int kGroupsPerPass = 2;
 
-// Shared-memory layout for NT threads, row_cap rows a slot (a.row_cap; a.ucap says
-// the same of dynamic batches).  K: floats per output corner.  own_palette: with
+// Shared-memory layout for NT threads, row_cap rows a slot (a.row_cap where batches
+// may hold more vertices than rows, else a.ucap).  K: floats per output corner.  own_palette: with
 // room for the skinning palette.
 __host__ __device__ inline ReuseLayout reuse_layout(int dedup, int shader, const DrawArgs& a, uint32_t NT,
                                                     uint32_t row_cap, bool own_palette) {

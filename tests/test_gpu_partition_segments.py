@@ -40,7 +40,7 @@ MESHES = {"grid": lambda T: mg.grid_mesh(220).indices[: 3 * T], "random": lambda
     (72960, 16, 341, 32), (72928, 16, 341, 32),  # windows of 32: warps from 2,280 segments on, and one less
     (72960, 3, 1365, 32), (91200, 256, 1, 32),
     (90001, 256, 341, 63), (90001, 64, 64, 33), (40001, 20, 80, 20), (40001, 256, 341, 128), (40001, 256, 341, 129),
-    (95000, 4096, 1365, 100), (95000, 3, 1, 40),
+    (95000, 4096, 1365, 100), (95000, 3, 1, 40), (95000, 4096, 1365, 256), (95000, 768, 256, 256), (95000, 767, 256, 256),
     (16384, 256, 341, 1), (16385, 256, 341, 1), (33333, 4, 7, 2),  # either side of the count by one block
 ])
 @pytest.mark.parametrize("kept", [False, True])
