@@ -2,7 +2,7 @@
 // static batch, persistent warps walking the batches with a grid stride.  The
 // per-batch work is warp_vote_batch (gp_warp_body.cuh): a chain of ~10 rounds of
 // votes, scattered row loads and shuffles per three batches, bound by the issue
-// of its instructions and the rows' latency.  1.09M triangles, S = 96: 49 us;
+// of its instructions and the rows' latency.  1.09M triangles, S = 96: 45 us;
 // written and stored round by round, 56.  The bound of 256 threads lets the compiler
 // choose 80 registers (24 warps an SM; 48 with the envelope shader): at 64 or 48 the
 // spills cost more (60 us), without it the kernel takes 140 (66 us), and asking for
@@ -82,8 +82,9 @@ static const void* warp_kernel_ptr(int shader, uint32_t batch_idx) {
 int warp_kernel_blocks_per_sm(int shader, int warps_per_block, uint32_t batch_idx) {
   const void* fn = warp_kernel_ptr(shader, batch_idx);
   const size_t smem = warp_kernel_smem(shader, warps_per_block, batch_idx);
+  // (no carveout for shared memory: what the blocks leave caches the rows; 7.2M triangles, S = 96 247 us against
+  // 291, S = 255 262 against 320)
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, warps_per_block * 32, smem) != cudaSuccess) return 1;
   return nb > 0 ? nb : 1;
